@@ -638,16 +638,21 @@ ppf_correct_ws_kernel(const TIn *__restrict__ raw, void *__restrict__ corr, cons
 }
 
 // Zero the padding of the planar layout that the fused kernel does not cover:
-// inputs [I, I_pad) and spectra [ceil16(S), S_pad) of every (subband, channel, plane).
-__global__ void planar_pad_kernel(unsigned short *__restrict__ corr, long long n_rows, int I, int I_pad, int S16,
-                                  int S_pad)
+// inputs [I, I_pad) and spectra [S16, s_out) of every (subband, channel, plane),
+// one plane per block in 16-byte stores. Bound by the bytes written: a plane's
+// padded inputs are one contiguous run (rows are in_row 16-byte words), the
+// padded spectra `gap` words at the end of each other row. 50 stations, 6144
+// channels, 700 spectra, split FP16 (415 MB of zeros): 59 us; a 64-thread block
+// per row, most of them with nothing to write, took 1382 us.
+__global__ void __launch_bounds__(256) planar_pad_kernel(uint4 *__restrict__ corr, int I, int I_pad, int in_row, int gap)
 {
-    const long long row = blockIdx.x;               // (sb, c, plane, i) flattened
-    if (row >= n_rows) return;
-    const int i = (int)(row % I_pad);
-    unsigned short *r = corr + row * S_pad;
-    const int from = (i >= I) ? 0 : S16;
-    for (int s = from + threadIdx.x; s < S_pad; s += blockDim.x) r[s] = 0;
+    uint4 *plane = corr + (long long)blockIdx.x * I_pad * in_row;
+    const int tail = (I_pad - I) * in_row;
+    for (int q = threadIdx.x; q < tail; q += blockDim.x) plane[(long long)I * in_row + q] = make_uint4(0, 0, 0, 0);
+    for (int q = threadIdx.x; q < I * gap; q += blockDim.x) {
+        const int row = q / gap;
+        plane[(long long)row * in_row + (in_row - gap) + (q - row * gap)] = make_uint4(0, 0, 0, 0);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -931,12 +936,13 @@ ppf_correct_ws256_kernel(const TIn *__restrict__ raw, void *__restrict__ corr, c
 cudaError_t planar_pad(const Handle &h, void *corr, int out, int S16, int s_out, cudaStream_t st)
 {
     if (h.I_pad <= h.I && s_out <= S16) return cudaSuccess;
-    const long long rows = (long long)h.p.n_subbands * h.p.n_channels * (out == 4 ? 4 : 2) * h.I_pad;
-    if (rows > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    // zero bits are zero in either element size: FP32 rows are twice as many 16-bit words
-    const int w = out == 5 ? 2 : 1;
-    planar_pad_kernel<<<(unsigned)rows, 64, 0, st>>>(reinterpret_cast<unsigned short *>(corr), rows, h.I, h.I_pad,
-                                                      w * S16, w * s_out);
+    const long long planes = (long long)h.p.n_subbands * h.p.n_channels * (out == 4 ? 4 : 2);
+    // S16 and s_out are multiples of 16 values, so rows and gaps are whole 16-byte words
+    const int per = out == 5 ? 4 : 8;
+    if (planes > 0x7fffffffLL || (long long)h.I_pad * (s_out / per) > 0x7fffffffLL)
+        return cudaErrorInvalidConfiguration;
+    planar_pad_kernel<<<(unsigned)planes, 256, 0, st>>>(reinterpret_cast<uint4 *>(corr), h.I, h.I_pad, s_out / per,
+                                                         max(s_out - S16, 0) / per);
     return cudaGetLastError();
 }
 
