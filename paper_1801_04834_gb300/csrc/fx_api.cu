@@ -47,7 +47,7 @@ namespace fxi {
 bool xstage_supported(const Handle &h)
 {
     if (h.p.precision == FX_F32) return true;
-    if (h.p.precision == FX_TF32_SPLIT) return xtf32_supported(h.I_pad, h.S_pad);
+    if (h.p.precision == FX_TF32_SPLIT) return xsplit_supported(h.I_pad);
     int rl, stg;
     unsigned sb;
     return xtc_plan(h, &rl, &stg, &sb);
@@ -56,8 +56,9 @@ bool xstage_supported(const Handle &h)
 cudaError_t launch_xstage(const Handle &h, const void *corr, float2 *vis, cudaStream_t st, bool accumulate)
 {
     switch (h.p.precision) {
-    case FX_F32: return launch_xcorr_f32(h, static_cast<const float2 *>(corr), vis, st, accumulate);
-    case FX_TF32_SPLIT: return launch_xcorr_tf32(h, static_cast<const float *>(corr), vis, st, accumulate);
+    case FX_F32:
+        return launch_xcorr_f32(h, static_cast<const float2 *>(corr), vis, st, accumulate);
+    case FX_TF32_SPLIT: return launch_xcorr_split(h, static_cast<const float *>(corr), vis, st);
     default: return launch_xcorr_tc(h, corr, vis, st, accumulate);
     }
 }
@@ -527,6 +528,14 @@ extern "C" fx_status fx_correct_correlate_backward(fx_handle *h, const float *d_
                         who);
 }
 
+// The correlations inside the moving-delay adjoint: its FP64 gradients keep the
+// rounding of these two forms (xcorr_tf32.cu)
+static cudaError_t adjoint_xstage(const fx_handle &h, const void *corr, float2 *vis, cudaStream_t s)
+{
+    return h.p.precision == FX_F32 ? fxi::launch_xcorr_f32(h, static_cast<const float2 *>(corr), vis, s)
+                                   : fxi::launch_xcorr_tf32(h, static_cast<const float *>(corr), vis, s);
+}
+
 extern "C" fx_status fx_correct_correlate_backward_interp(
     fx_handle *h, const float *d_chan, const double *d_delay_begin, const double *d_delay_end,
     const float *d_bandpass, const float *d_gains, const float *d_grad_vis, void *d_work_corr, float *d_work_vis,
@@ -552,9 +561,9 @@ extern "C" fx_status fx_correct_correlate_backward_interp(
     cudaError_t e = fxi::launch_phase_table(*h, d_delay_begin, d_delay_end, s);
     if (e == cudaSuccess)   // the corrected block with unit gains: Y
         e = fxi::launch_correct(*h, reinterpret_cast<const float2 *>(d_chan), d_bandpass, nullptr, d_work_corr, s);
-    if (e == cudaSuccess) e = fxi::launch_xstage(*h, d_work_corr, K, s);              // K = sum Y Y^H
+    if (e == cudaSuccess) e = adjoint_xstage(*h, d_work_corr, K, s);                  // K = sum Y Y^H
     if (e == cudaSuccess) e = fxi::launch_weight_spectra(*h, d_work_corr, s);         // Y sqrt(s/S)
-    if (e == cudaSuccess) e = fxi::launch_xstage(*h, d_work_corr, M1, s);             // M1 = sum (s/S) Y Y^H
+    if (e == cudaSuccess) e = adjoint_xstage(*h, d_work_corr, M1, s);                 // M1 = sum (s/S) Y Y^H
     if (e == cudaSuccess)
         e = fxi::launch_adjoint_interp(*h, K, M1, reinterpret_cast<const float2 *>(d_grad_vis),
                                        reinterpret_cast<const float2 *>(d_gains),

@@ -103,10 +103,15 @@ cudaError_t launch_beamform_incoherent(const Handle &h, const void *corr, const 
 cudaError_t launch_beamform(const Handle &h, const void *corr, int n_beams, const double *delays,
                             const float *weights, int mode, int tint, float *out, cudaStream_t st);
 
-// xcorr_tf32.cu (FX_TF32_SPLIT)
-bool xtf32_supported(int I_pad, int S_pad);
-cudaError_t launch_xcorr_tf32(const Handle &h, const float *corr, float2 *vis, cudaStream_t st,
-                             bool accumulate = false);    // accumulate: add to vis
+// xcorr_split.cu (FX_TF32_SPLIT, and FX_F32 where xf32_on_tensor_cores)
+bool xsplit_supported(int I_pad);
+cudaError_t launch_xcorr_split(const Handle &h, const float *corr, float2 *vis, cudaStream_t st);
+bool xf32_on_tensor_cores(const Handle &h);   // FX_F32: this form rather than the CUDA-core one
+cudaError_t launch_xcorr_f32_tc(const Handle &h, const float2 *corr, float2 *vis, cudaStream_t st,
+                                bool accumulate = false);   // accumulate: add to vis
+
+// xcorr_tf32.cu (FX_TF32_SPLIT operands, every product formed: the moving-delay adjoint)
+cudaError_t launch_xcorr_tf32(const Handle &h, const float *corr, float2 *vis, cudaStream_t st);
 
 // probe.cu
 cudaError_t launch_ffma_probe(int iterations, int blocks, float *sink, cudaStream_t st);

@@ -1,5 +1,10 @@
-// xcorr_tf32.cu -- FP32-accurate X-stage on the tcgen05 tensor cores, any
-// station count: FP32 corrected samples split in the kernel into hi + lo,
+// xcorr_tf32.cu -- FP32-accurate correlation on the tcgen05 tensor cores with
+// every product formed, any station count: the X-stage of the moving-delay
+// adjoint, whose delay gradients are returned in FP64 and have to stay what
+// they were, to the last bits of the sums they are made of (xcorr_split.cu,
+// which forms half the products of a diagonal tile and is the X-stage of every
+// other call, rounds differently by about 1e-6). FP32 corrected samples split
+// in the kernel into hi + lo,
 // V ~ hi hi' + hi lo' + lo hi' (lo lo' dropped), the main term hi hi' as TF32
 // MMAs and the two cross terms as BF16 MMAs, FP32 accumulation in TMEM, chunk
 // sums added in IEEE FP32.
@@ -126,12 +131,12 @@ struct T3Params {
     unsigned stage_bytes;
     unsigned a_off;           // byte offset of the B region when an A region precedes it
     int no_tma;               // failure-detection test hook: issue no loads
-    int accumulate;           // add every chunk to vis (also the first)
 };
 
 __device__ __forceinline__ bool t3wait(unsigned bar, unsigned parity, volatile int *abort_flag, const T3Params &P,
                                        int code)
 {
+    if (mbar_try_wait(bar, parity)) return true;
     const long long t0 = clock64();
     while (!mbar_try_wait(bar, parity)) {
         if (*abort_flag) return false;
@@ -144,6 +149,22 @@ __device__ __forceinline__ bool t3wait(unsigned bar, unsigned parity, volatile i
     }
     return true;
 }
+
+// Position in the ring of stages: slot and the parity of its current use, stepped
+// without a division by the run-time depth (64-bit divisions, several per stage
+// and role: 76 stations x 2048 channels x 768 spectra 1.55 ms with them, 1.37
+// without).
+struct Ring {
+    int i = 0;
+    unsigned ph = 0;
+    __device__ __forceinline__ void step(int depth)
+    {
+        if (++i == depth) {
+            i = 0;
+            ph ^= 1u;
+        }
+    }
+};
 
 // Shared-memory matrix descriptor: K-major, 64-byte swizzle (8-row atoms of
 // 512 bytes, SBO = 512), LBO unused for this layout, descriptor version 1.
@@ -300,7 +321,8 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_tf32_kernel(const __grid_
     if (warp == 0) {
         // ================= TMA producer =================
         if (lane == 0) {
-            long long it = 0;
+            Ring ring;
+            int filled = 0;                             // stages with a copy issued, up to the ring's depth
             bool ok = true;
             for (long long w = blockIdx.x; w < P.n_items && ok; w += gridDim.x) {
                 const int4 itm = P.items[(int)(w % P.ipc)];
@@ -310,13 +332,14 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_tf32_kernel(const __grid_
                 const bool full_diag = diag && n == 128;
                 const unsigned boff = diag ? 0u : P.a_off;
                 const unsigned tx = (diag ? 0u : 2u * kT3APlane) + 2u * (unsigned)n * kT3RowBytes;
-                for (int kc = 0; kc < P.nk; ++kc, ++it) {
-                    const int s = (int)(it % P.stages);
-                    if (!t3wait(empty_bar(s), (unsigned)((it / P.stages) & 1) ^ 1u, abort_flag, P, 1)) {
+                for (int kc = 0; kc < P.nk; ++kc, ring.step(P.stages)) {
+                    const int s = ring.i;
+                    if (!t3wait(empty_bar(s), ring.ph ^ 1u, abort_flag, P, 1)) {
                         ok = false;
                         break;
                     }
                     if (P.no_tma) continue;
+                    filled = min(filled + 1, P.stages);
                     mbar_arrive_expect_tx(full_bar(s), tx);
                     const unsigned dst = tiles_u32 + (unsigned)s * P.stage_bytes;
                     for (int pl = 0; pl < 2; ++pl) {
@@ -334,16 +357,21 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_tf32_kernel(const __grid_
                     }
                 }
             }
-            if (!ok && !P.no_tma) {
-                const long long first = it > P.stages ? it - P.stages : 0;
-                for (long long u = first; u < it; ++u)
-                    drain_wait(full_bar((int)(u % P.stages)), (unsigned)((u / P.stages) & 1), P.timeout_cycles);
+            if (!ok) {                                  // wait for the copies of the ring's last uses
+                for (int u = 0; u < filled; ++u) {
+                    if (--ring.i < 0) {
+                        ring.i = P.stages - 1;
+                        ring.ph ^= 1u;
+                    }
+                    drain_wait(full_bar(ring.i), ring.ph, P.timeout_cycles);
+                }
             }
         }
     } else if (warp == 1) {
         // ================= MMA issuer =================
         if (lane == 0) {
-            long long it = 0, acc_it = 0;
+            Ring ring;
+            unsigned acc_it = 0;
             bool ok = true, issued = false;
             for (long long w = blockIdx.x; w < P.n_items && ok; w += gridDim.x) {
                 const int4 itm = P.items[(int)(w % P.ipc)];
@@ -355,15 +383,15 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_tf32_kernel(const __grid_
                 const unsigned idesc_bf = make_idesc(1u, 2 * n, false);
                 for (int ch = 0; ch < n_chunks && ok; ++ch, ++acc_it) {
                     const int ab = (int)(acc_it & 1);
-                    if (!t3wait(acce_bar(ab), (unsigned)((acc_it >> 1) & 1) ^ 1u, abort_flag, P, 2)) {
+                    if (!t3wait(acce_bar(ab), ((acc_it >> 1) & 1u) ^ 1u, abort_flag, P, 2)) {
                         ok = false;
                         break;
                     }
                     tc_fence_after();
                     const unsigned d = tmem_base + (unsigned)(ab * kT3AccCols);
-                    for (int kc = 0; kc < P.chunk; ++kc, ++it) {
-                        const int s = (int)(it % P.stages);
-                        if (!t3wait(conv_bar(s), (unsigned)((it / P.stages) & 1), abort_flag, P, 2)) {
+                    for (int kc = 0; kc < P.chunk; ++kc, ring.step(P.stages)) {
+                        const int s = ring.i;
+                        if (!t3wait(conv_bar(s), ring.ph, abort_flag, P, 2)) {
                             ok = false;
                             break;
                         }
@@ -406,16 +434,16 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_tf32_kernel(const __grid_
     } else if (warp >= kT3ConvWarp0) {
         // ================= converter (warps 10..13) =================
         const int ct = threadIdx.x - kT3ConvWarp0 * 32; // 0..127
-        long long it = 0;
+        Ring ring;
         bool ok = true;
         for (long long w = blockIdx.x; w < P.n_items && ok; w += gridDim.x) {
             const int4 itm = P.items[(int)(w % P.ipc)];
             const int n = itm.z;
             const bool diag = itm.w != 0;
             const unsigned pitch = (unsigned)n * kT3RowBytes;
-            for (int kc = 0; kc < P.nk; ++kc, ++it) {
-                const int s = (int)(it % P.stages);
-                const bool got = t3wait(full_bar(s), (unsigned)((it / P.stages) & 1), abort_flag, P, 4);
+            for (int kc = 0; kc < P.nk; ++kc, ring.step(P.stages)) {
+                const int s = ring.i;
+                const bool got = t3wait(full_bar(s), ring.ph, abort_flag, P, 4);
                 if (!__all_sync(0xffffffffu, got)) {
                     ok = false;
                     break;
@@ -434,7 +462,7 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_tf32_kernel(const __grid_
         // ================= epilogue (warps 2..9) =================
         const int qd = warp & 3;                        // TMEM lane quadrant
         const int half = (warp - 2) >> 2;               // which 32-column groups
-        long long acc_it = 0;
+        unsigned acc_it = 0;
         bool live = true;
         for (long long w = blockIdx.x; w < P.n_items && live; w += gridDim.x) {
             const int4 itm = P.items[(int)(w % P.ipc)];
@@ -447,13 +475,13 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_tf32_kernel(const __grid_
             float2 *vrow = P.vis + gch * P.B * 4;
             for (int ch = 0; ch < n_chunks; ++ch, ++acc_it) {
                 const int ab = (int)(acc_it & 1);
-                const bool got = t3wait(accf_bar(ab), (unsigned)((acc_it >> 1) & 1), abort_flag, P, 3);
+                const bool got = t3wait(accf_bar(ab), (acc_it >> 1) & 1u, abort_flag, P, 3);
                 if (!__all_sync(0xffffffffu, got)) {
                     live = false;
                     break;
                 }
                 tc_fence_after();
-                const bool store = (ch == 0) && !P.accumulate;
+                const bool store = ch == 0;
                 const unsigned t = tmem_base + ((unsigned)(32 * qd) << 16) + (unsigned)(ab * kT3AccCols);
                 if (i_warp_min < P.N) {
                     for (int cc = 2 * half; cc < ncc; cc += 4) {
@@ -552,13 +580,7 @@ bool t3_plan(int I_pad, int NT, T3Plan &pl)
 
 }  // namespace
 
-bool xtf32_supported(int I_pad, int S_pad)
-{
-    T3Plan pl;
-    return S_pad % (kT3K * 4) == 0 && t3_plan(I_pad, 64, pl);
-}
-
-cudaError_t launch_xcorr_tf32(const Handle &h, const float *corr, float2 *vis, cudaStream_t st, bool accumulate)
+cudaError_t launch_xcorr_tf32(const Handle &h, const float *corr, float2 *vis, cudaStream_t st)
 {
     EncodeTiledFn enc = t3_encode_fn();
     if (!enc) return cudaErrorNotSupported;
@@ -597,7 +619,6 @@ cudaError_t launch_xcorr_tf32(const Handle &h, const float *corr, float2 *vis, c
     P.a_off = pl.a_off;
     P.timeout_cycles = h.tc_timeout_cycles;
     P.no_tma = h.tc_test_no_tma;
-    P.accumulate = accumulate ? 1 : 0;
     const size_t smem = 1024 + (size_t)pl.stages * pl.stage_bytes + 8 * kT3Bars + 16;
     cudaError_t e = cudaFuncSetAttribute(xcorr_tf32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
