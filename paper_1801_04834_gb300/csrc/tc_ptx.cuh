@@ -35,6 +35,29 @@ __device__ __forceinline__ bool mbar_try_wait(unsigned bar, unsigned parity)
     return ok != 0;
 }
 
+// Position in a ring of buffers: slot and the parity of its current use, stepped
+// without a division. Dividing a 64-bit counter by the run-time depth, several
+// times per stage and role, took longer than a stage's MMAs (FP32-accurate
+// X-stage, 64 stations x 1280 channels x 3072 spectra: 1.39 against 1.01 ms).
+struct Ring {
+    int i = 0;
+    unsigned ph = 0;
+    __device__ __forceinline__ void step(int depth)
+    {
+        if (++i == depth) {
+            i = 0;
+            ph ^= 1u;
+        }
+    }
+    __device__ __forceinline__ void back(int depth)
+    {
+        if (--i < 0) {
+            i = depth - 1;
+            ph ^= 1u;
+        }
+    }
+};
+
 // Bounded wait used while draining after an abort (ignores the abort flag).
 __device__ __forceinline__ void drain_wait(unsigned bar, unsigned parity, long long budget)
 {

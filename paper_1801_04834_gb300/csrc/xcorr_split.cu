@@ -169,21 +169,6 @@ __device__ __forceinline__ bool t3wait(unsigned bar, unsigned parity, volatile i
     return true;
 }
 
-// Position in a ring of buffers: slot and the parity of its current use, stepped
-// without a division (64-bit divisions by the run-time depth, several per
-// stage and role, took longer than the stage's MMAs: 1.39 against 1.01 ms).
-struct Ring {
-    int i = 0;
-    unsigned ph = 0;
-    __device__ __forceinline__ void step(int depth)
-    {
-        if (++i == depth) {
-            i = 0;
-            ph ^= 1u;
-        }
-    }
-};
-
 // Shared-memory matrix descriptor: K-major, 64-byte swizzle (8-row atoms of
 // 512 bytes, SBO = 512), LBO unused for this layout, descriptor version 1.
 __device__ __forceinline__ unsigned long long sdesc64(unsigned addr)
@@ -524,10 +509,7 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_split_kernel(const __grid
                 }
                 if (!ok) {                             // wait for the copies of the ring's last uses
                     for (int u = 0; u < filled; ++u) {
-                        if (--ring.i < 0) {
-                            ring.i = P.lands - 1;
-                            ring.ph ^= 1u;
-                        }
+                        ring.back(P.lands);
                         drain_wait(full_bar(ring.i), ring.ph, P.timeout_cycles);
                     }
                 }

@@ -116,6 +116,7 @@ struct Item {
 __device__ __forceinline__ bool wait_bounded(unsigned bar, unsigned parity, volatile int *abort_flag,
                                              const TcCommon &a, int code)
 {
+    if (mbar_try_wait(bar, parity)) return true;
     const long long t0 = clock64();
     while (!mbar_try_wait(bar, parity)) {
         if (*abort_flag) return false;
@@ -241,7 +242,8 @@ __global__ void __launch_bounds__(kThreads, 1) xcorr_tc_kernel(const __grid_cons
     if (warp == 0) {
         // ================= TMA producer =================
         if (lane == 0) {
-            long long it = 0;
+            Ring ring;
+            int filled = 0;                             // stages with a copy issued, up to the ring's depth
             bool ok = true;
             for (long long w = blockIdx.x; w < a.n_items && ok; w += gridDim.x) {
                 const Item itm = decode(P, w);
@@ -250,11 +252,11 @@ __global__ void __launch_bounds__(kThreads, 1) xcorr_tc_kernel(const __grid_cons
                 item_cols(P, J, itm, row0, col0, ncols);
                 const bool diag = (col0 == row0);
                 const unsigned tx = (unsigned)a.planes * 128u * (J.ra + (diag ? 0 : a.NT));
-                for (int kc = 0; kc < J.nk; ++kc, ++it) {
-                    const int s = (int)(it % a.stages);
-                    const unsigned ph = (unsigned)((it / a.stages) & 1);
-                    if (!wait_bounded(empty_bar(s), ph ^ 1u, abort_flag, a, 1)) { ok = false; break; }
+                for (int kc = 0; kc < J.nk; ++kc, ring.step(a.stages)) {
+                    const int s = ring.i;
+                    if (!wait_bounded(empty_bar(s), ring.ph ^ 1u, abort_flag, a, 1)) { ok = false; break; }
                     if (a.no_tma) continue;
+                    filled = min(filled + 1, a.stages);
                     mbar_arrive_expect_tx(full_bar(s), tx);
                     const unsigned dst = tiles_u32 + (unsigned)s * a.stage_bytes;
                     for (int pl = 0; pl < a.planes; ++pl) {
@@ -266,17 +268,21 @@ __global__ void __launch_bounds__(kThreads, 1) xcorr_tc_kernel(const __grid_cons
                     }
                 }
             }
-            if (!ok && !a.no_tma) {
-                // drain: the last `stages` loads issued may still be in flight
-                const long long first = it > a.stages ? it - a.stages : 0;
-                for (long long u = first; u < it; ++u)
-                    drain_wait(full_bar((int)(u % a.stages)), (unsigned)((u / a.stages) & 1), a.timeout_cycles);
+            if (!ok) {                                  // wait for the copies of the ring's last uses
+                for (int u = 0; u < filled; ++u) {
+                    ring.back(a.stages);
+                    drain_wait(full_bar(ring.i), ring.ph, a.timeout_cycles);
+                }
             }
         }
     } else if (warp == 1) {
         // ================= MMA issuer =================
         if (lane == 0) {
-            long long it = 0, acc_it = 0;
+            Ring ring, accs;
+            // descriptors are built once; a plane, stage or K-step further on is an addition
+            // in 16-byte units (one thread issues every MMA)
+            const unsigned long long desc0 = smem_desc(tiles_u32);
+            const unsigned ap = a_plane >> 4;
             bool ok = true, issued = false;
             for (long long w = blockIdx.x; w < a.n_items && ok; w += gridDim.x) {
                 const Item itm = decode(P, w);
@@ -287,40 +293,38 @@ __global__ void __launch_bounds__(kThreads, 1) xcorr_tc_kernel(const __grid_cons
                 const unsigned idesc = make_idesc(a.bf16, ncols, false);
                 const unsigned idesc_neg = make_idesc(a.bf16, ncols, true);
                 const int clen = a.chunk > 0 ? a.chunk : J.nk;   // stages per accumulator chain
-                for (int k0 = 0; k0 < J.nk && ok; k0 += clen, ++acc_it) {
-                    const int ab = (int)(acc_it % a.nacc);
-                    const unsigned aph = (unsigned)((acc_it / a.nacc) & 1);
-                    if (!wait_bounded(acce_bar(ab), aph ^ 1u, abort_flag, a, 2)) { ok = false; break; }
+                const unsigned bo = diag ? 0u : a_region >> 4, bp = (diag ? a_plane : b_plane) >> 4;
+                for (int k0 = 0; k0 < J.nk && ok; k0 += clen, accs.step(a.nacc)) {
+                    const int ab = accs.i;
+                    if (!wait_bounded(acce_bar(ab), accs.ph ^ 1u, abort_flag, a, 2)) { ok = false; break; }
                     tc_fence_after();
                     const unsigned d_re = tmem_base + (unsigned)(ab * a.acc_stride);
                     const unsigned d_im = d_re + (unsigned)a.ncm;
                     const int k1 = min(J.nk, k0 + clen);
-                    for (int kc = k0; kc < k1; ++kc, ++it) {
-                        const int s = (int)(it % a.stages);
-                        const unsigned ph = (unsigned)((it / a.stages) & 1);
-                        if (!wait_bounded(full_bar(s), ph, abort_flag, a, 2)) { ok = false; break; }
+                    for (int kc = k0; kc < k1; ++kc, ring.step(a.stages)) {
+                        const int s = ring.i;
+                        if (!wait_bounded(full_bar(s), ring.ph, abort_flag, a, 2)) { ok = false; break; }
                         tc_fence_after();
-                        const unsigned tile = tiles_u32 + (unsigned)s * a.stage_bytes;
-                        const unsigned btile = diag ? tile : tile + a_region;
-                        const unsigned bpl = diag ? a_plane : b_plane;
+                        const unsigned long long ta = desc0 + (unsigned)s * (a.stage_bytes >> 4);
+                        const unsigned long long tb = ta + bo;
 #pragma unroll
                         for (int kk = 0; kk < kBK / 16; ++kk) {
                             const unsigned acc = (kc != k0 || kk) ? 1u : 0u;
                             // A operand rows = the row block, B operand rows = the column block
-                            const unsigned long long ar0 = smem_desc(tile + 0 * a_plane + kk * 32);
-                            const unsigned long long aj0 = smem_desc(tile + 1 * a_plane + kk * 32);
-                            const unsigned long long br0 = smem_desc(btile + 0 * bpl + kk * 32);
-                            const unsigned long long bj0 = smem_desc(btile + 1 * bpl + kk * 32);
+                            const unsigned long long ar0 = ta + kk * 2;
+                            const unsigned long long aj0 = ta + ap + kk * 2;
+                            const unsigned long long br0 = tb + kk * 2;
+                            const unsigned long long bj0 = tb + bp + kk * 2;
                             if (a.planes == 2) {
                                 mma_f16(d_re, ar0, br0, idesc, acc);
                                 mma_f16(d_re, aj0, bj0, idesc, 1u);
                                 mma_f16(d_im, aj0, br0, idesc, acc);
                                 mma_f16(d_im, ar0, bj0, idesc_neg, 1u);
                             } else {
-                                const unsigned long long ar1 = smem_desc(tile + 2 * a_plane + kk * 32);
-                                const unsigned long long aj1 = smem_desc(tile + 3 * a_plane + kk * 32);
-                                const unsigned long long br1 = smem_desc(btile + 2 * bpl + kk * 32);
-                                const unsigned long long bj1 = smem_desc(btile + 3 * bpl + kk * 32);
+                                const unsigned long long ar1 = ta + 2 * ap + kk * 2;
+                                const unsigned long long aj1 = ta + 3 * ap + kk * 2;
+                                const unsigned long long br1 = tb + 2 * bp + kk * 2;
+                                const unsigned long long bj1 = tb + 3 * bp + kk * 2;
                                 // (hi, hi)
                                 mma_f16(d_re, ar0, br0, idesc, acc);
                                 mma_f16(d_re, aj0, bj0, idesc, 1u);
@@ -354,7 +358,7 @@ __global__ void __launch_bounds__(kThreads, 1) xcorr_tc_kernel(const __grid_cons
     } else {
         // ================= epilogue (warps 2..5) =================
         const int qd = warp & 3;                      // TMEM lane quadrant of this warp
-        long long acc_it = 0;
+        Ring accs;
         bool live = true;
         for (long long w = blockIdx.x; w < a.n_items && live; w += gridDim.x) {
             const Item itm = decode(P, w);
@@ -367,10 +371,9 @@ __global__ void __launch_bounds__(kThreads, 1) xcorr_tc_kernel(const __grid_cons
             const int i_warp_min = (row0 + 32 * qd) >> 1;
             const unsigned lane_off = (unsigned)(32 * qd) << 16;
             float2 *vrow = J.vis + itm.gch * J.B * 4;
-            for (int k0 = 0; k0 < J.nk; k0 += clen, ++acc_it) {
-                const int ab = (int)(acc_it % a.nacc);
-                const unsigned aph = (unsigned)((acc_it / a.nacc) & 1);
-                const bool got = wait_bounded(accf_bar(ab), aph, abort_flag, a, 3);
+            for (int k0 = 0; k0 < J.nk; k0 += clen, accs.step(a.nacc)) {
+                const int ab = accs.i;
+                const bool got = wait_bounded(accf_bar(ab), accs.ph, abort_flag, a, 3);
                 if (!__all_sync(0xffffffffu, got)) {   // warp-uniform exit
                     live = false;
                     break;

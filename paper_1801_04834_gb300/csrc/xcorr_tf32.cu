@@ -150,22 +150,6 @@ __device__ __forceinline__ bool t3wait(unsigned bar, unsigned parity, volatile i
     return true;
 }
 
-// Position in the ring of stages: slot and the parity of its current use, stepped
-// without a division by the run-time depth (64-bit divisions, several per stage
-// and role: 76 stations x 2048 channels x 768 spectra 1.55 ms with them, 1.37
-// without).
-struct Ring {
-    int i = 0;
-    unsigned ph = 0;
-    __device__ __forceinline__ void step(int depth)
-    {
-        if (++i == depth) {
-            i = 0;
-            ph ^= 1u;
-        }
-    }
-};
-
 // Shared-memory matrix descriptor: K-major, 64-byte swizzle (8-row atoms of
 // 512 bytes, SBO = 512), LBO unused for this layout, descriptor version 1.
 __device__ __forceinline__ unsigned long long sdesc64(unsigned addr)
@@ -359,10 +343,7 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_tf32_kernel(const __grid_
             }
             if (!ok) {                                  // wait for the copies of the ring's last uses
                 for (int u = 0; u < filled; ++u) {
-                    if (--ring.i < 0) {
-                        ring.i = P.stages - 1;
-                        ring.ph ^= 1u;
-                    }
+                    ring.back(P.stages);
                     drain_wait(full_bar(ring.i), ring.ph, P.timeout_cycles);
                 }
             }
