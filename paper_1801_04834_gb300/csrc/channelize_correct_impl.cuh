@@ -63,16 +63,45 @@ constexpr size_t fused_smem_bytes()
     return ppf_smem_bytes<C, TIn>() + (size_t)kRound * Cfg::NPC * kPols * fused_phc<C>() * sizeof(float2);
 }
 
-__device__ __forceinline__ unsigned short to_bits(float x, int out)
+// two values as 16-bit operands (OUT 3 BF16, else FP16), the first in the low half
+template <int OUT>
+__device__ __forceinline__ unsigned pack16(float a, float b)
 {
-    if (out == 3) return __bfloat16_as_ushort(__float2bfloat16_rn(x));
-    return __half_as_ushort(__float2half_rn(x));
+    if constexpr (OUT == 3) {
+        const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+        return *reinterpret_cast<const unsigned *>(&v);
+    } else {
+        const __half2 v = __floats2half2_rn(a, b);
+        return *reinterpret_cast<const unsigned *>(&v);
+    }
 }
 
-// lo part of split FP16: x - hi rounded to FP16, hi = the FP16 bits of x
-__device__ __forceinline__ unsigned short lo_bits16(float x, unsigned short hi)
+// lo parts of split FP16: x - hi rounded to FP16, hi = pack16's halves
+__device__ __forceinline__ unsigned pack16_lo(float a, float b, unsigned hi)
 {
-    return __half_as_ushort(__float2half_rn(x - __half2float(__ushort_as_half(hi))));
+    const float2 h = __half22float2(*reinterpret_cast<const __half2 *>(&hi));
+    return pack16<4>(a - h.x, b - h.y);
+}
+
+// Two adjacent spectra of one (channel, input) into the planar planes, o = the
+// offset of the first in plane 0 (OUT 2 FP16, 3 BF16, 4 split FP16, 5 FP32).
+template <int OUT>
+__device__ __forceinline__ void store_planar(void *corr, long long o, long long pstride, float2 ya, float2 yb)
+{
+    if constexpr (OUT == 5) {
+        float *out = reinterpret_cast<float *>(corr) + o;
+        *reinterpret_cast<float2 *>(out) = make_float2(ya.x, yb.x);
+        *reinterpret_cast<float2 *>(out + pstride) = make_float2(ya.y, yb.y);
+    } else {
+        unsigned short *out = reinterpret_cast<unsigned short *>(corr) + o;
+        const unsigned re = pack16<OUT>(ya.x, yb.x), im = pack16<OUT>(ya.y, yb.y);
+        *reinterpret_cast<unsigned *>(out) = re;
+        *reinterpret_cast<unsigned *>(out + pstride) = im;
+        if constexpr (OUT == 4) {
+            *reinterpret_cast<unsigned *>(out + 2 * pstride) = pack16_lo(ya.x, yb.x, re);
+            *reinterpret_cast<unsigned *>(out + 3 * pstride) = pack16_lo(ya.y, yb.y, im);
+        }
+    }
 }
 
 template <int C, int T, typename TIn, int OUT>
@@ -610,25 +639,7 @@ ppf_correct_ws_kernel(const TIn *__restrict__ raw, void *__restrict__ corr, cons
                             const int kout = k1 + R * ((k2 + R / 2) % R);
                             const float2 ya = va[k2], yb = vb[k2];
                             const long long o = base + (long long)kout * planes * pstride;
-                            if constexpr (OUT == 5) {
-                                float *out = reinterpret_cast<float *>(corr);
-                                *reinterpret_cast<float2 *>(out + o) = make_float2(ya.x, yb.x);
-                                *reinterpret_cast<float2 *>(out + o + pstride) = make_float2(ya.y, yb.y);
-                            } else {
-                                unsigned short *out = reinterpret_cast<unsigned short *>(corr);
-                                const unsigned short ra = to_bits(ya.x, OUT), ia = to_bits(ya.y, OUT);
-                                const unsigned short rb = to_bits(yb.x, OUT), ib = to_bits(yb.y, OUT);
-                                *reinterpret_cast<unsigned *>(out + o) = (unsigned)ra | ((unsigned)rb << 16);
-                                *reinterpret_cast<unsigned *>(out + o + pstride) = (unsigned)ia | ((unsigned)ib << 16);
-                                if constexpr (OUT == 4) {
-                                    const unsigned short lra = lo_bits16(ya.x, ra), lia = lo_bits16(ya.y, ia);
-                                    const unsigned short lrb = lo_bits16(yb.x, rb), lib = lo_bits16(yb.y, ib);
-                                    *reinterpret_cast<unsigned *>(out + o + 2 * pstride) =
-                                        (unsigned)lra | ((unsigned)lrb << 16);
-                                    *reinterpret_cast<unsigned *>(out + o + 3 * pstride) =
-                                        (unsigned)lia | ((unsigned)lib << 16);
-                                }
-                            }
+                            store_planar<OUT>(corr, o, pstride, ya, yb);
                         }
                     }
                 }
@@ -657,68 +668,84 @@ __global__ void __launch_bounds__(256) planar_pad_kernel(uint4 *__restrict__ cor
 
 // ---------------------------------------------------------------------------
 // Warp-specialised fused kernel for C = 256 with planar outputs (OUT = 2..5):
-// one CTA per (station, pol), 256 FIR threads (one channel each) and 256 FFT
-// threads in two groups of 128, one CTA per SM. A round's rows (16 spectra
-// of one input) fit twice in shared memory at this channel count only per
-// input; the CTAs of a station's two pols are neighbours in the grid and read
-// the same raw rows (the second read mostly from L2). FIR round b -> u[b & 1]
-// and the whole per-sample factor bandpass x gain x flag x exp(i phi) of its
-// 16 spectra (one __sincosf per channel and round, multiplied once by
-// bandpass x gain, then rotations by exp(i step) computed in FP32 from the
-// FP64-derived step; bandpass x gain is constant per channel within a CTA,
-// which serves one input) -> FULL[b & 1]. FFT group g takes the rounds
-// b = g mod 2 (row buffer g) with its own named barrier, so two rounds are in
-// FFT at once and each FFT thread has two transforms in flight per pass
-// (36.6 against 39.5 ms at the 8-bit workload with one group of 256): pass 1
-// (row = 16 lanes), transposed into P1[k1][n2][row] over u[g] after the
-// group's barrier, pass 2 with lane = spectrum (a half-warp per k1), so a
-// warp store is 2 x 32 bytes of planar rows.
+// one CTA per (station, pol) and SM, 256 FIR threads (one channel each) and 256
+// FFT threads in two groups of 128. A round's rows (16 spectra of one input) fit
+// twice in shared memory at this channel count only per input; the CTAs of a
+// station's two pols are neighbours in the grid and read the same raw rows (the
+// second read mostly from L2). FIR round b -> u[b & 1] -> FULL[b & 1]; FFT group
+// g takes the rounds b = g mod 2 (row buffer g) with its own named barrier, so
+// two rounds are in FFT at once.
+//
+// What bounds it: the FMA pipe with the register reads of its packed FMAs. The
+// FIR alone (16 warps, nothing else running) takes 2.0 ms of the 8-bit case below,
+// 0.64 of the pipe's rate in every instruction order tried, and the FFT's adds and
+// multiplies 1.4 ms at full rate, 3.4 ms together; more warps (20, 24) gain
+// nothing. So the design saves instructions and shared-memory traffic:
+//  * the phase factors come from the channel axis. f_k is linear in k, so for a
+//    spectrum s exp(i phi(k, s)) = e(k1, s) r(s)^m for k = k1 + 128 + 16 m: the
+//    FIR threads put one anchor e (16 x 16 per round, each the gain, flag and
+//    scale times one __sincosf) into a table, the phase-table kernel has left
+//    r(s) = exp(2 pi i (fs / 16) tau(s)) per station and spectrum, and an FFT
+//    thread steps from its anchor up and down eight channels each in registers.
+//    (One entry per channel and spectrum, rotated along time by the FIR threads,
+//    took a 70 KB table and a store and a load per output.)
+//  * pass 1 (row = 16 lanes) writes its results transposed, P1[k1][n2][row] over
+//    u[g] after the group's barrier; in pass 2 a thread takes two adjacent
+//    spectra of one k1, so P1 rows come in 16-byte loads and planar values leave
+//    in pairs (a warp store is 4 x 32 bytes of rows, FP32 4 x 64).
+//  * strides: FIR rows 264 (two rows' halves fall on both halves of the banks in
+//    pass 1), P1 rows 18 (even, for the 16-byte loads; eight n2 x two rows of a
+//    store on distinct banks).
+// 64 stations, 61 subbands of int8, 768 spectra, FP16 out: 4.45 -> 4.16 ms (2.2
+// TB/s of raw rows and operands); two row buffers instead of four 4.34 ms.
 struct Ws256 {
-    static constexpr int C = 256, R = 16, NF = 256;
-    static constexpr int ROW = C + 16;                  // FIR row stride (float2)
-    static constexpr int USZ = kRound * ROW;            // one row buffer: 16 spectra
-    static constexpr int RS = kRound + 1;               // P1 row stride
-    static constexpr int EJ = kRound + 1;               // phasor table: [C][EJ]
-    static constexpr int ESZ = C * EJ;
-    static_assert(R * R * RS <= USZ, "P1 fits over the row buffer");
+    static constexpr int C = 256, R = 16;
+    static constexpr int NF = C, NG = 128;              // FIR threads; FFT threads of a group
+    static constexpr int ALL = NF + 2 * NG;
+    static constexpr int ROW = C + 8;                   // FIR row stride (float2)
+    static constexpr int RS = kRound + 2;               // P1 row stride
+    static constexpr int USZ = R * R * RS > kRound * ROW ? R * R * RS : kRound * ROW;   // one buffer: 16 rows, then P1
+    static constexpr int TW = R + 2;                    // twiddle row: [n2][k1], even
+    static constexpr int ESZ = R * kRound;              // anchors [k1][spectrum] of a round
+    static constexpr int NB = 4;                        // row buffers
 };
 
 template <typename TIn>
 constexpr size_t ws256_smem_bytes()
 {
     using W = Ws256;
-    return (size_t)W::C * sizeof(float2) + 2ull * kRound * W::C * kPols * sizeof(TIn) +
-           (2ull * W::USZ + 2ull * W::ESZ + 2ull * W::C) * sizeof(float2) + 16;   // + 2 mbarriers
+    return 2ull * kRound * W::C * kPols * sizeof(TIn) +
+           ((size_t)W::NB * (W::USZ + W::ESZ) + (size_t)W::R * W::TW) * sizeof(float2) + W::C * sizeof(float2) + 16;   // + 2 mbarriers
 }
 
+__device__ __forceinline__ float2 conj2(float2 a) { return make_float2(a.x, -a.y); }
+
 template <int T, typename TIn, int OUT>
-__global__ void __launch_bounds__(2 * Ws256::NF, 1)
+__global__ void __launch_bounds__(Ws256::ALL, 1)
 ppf_correct_ws256_kernel(const TIn *__restrict__ raw, void *__restrict__ corr, const float *__restrict__ taps,
                          const float2 *__restrict__ twiddle, const float2 *__restrict__ phase,
-                         const float *__restrict__ bandpass, const float2 *__restrict__ gains, int N, int S,
-                         int I_pad, int s_out, float scale, int rounds_per_cta, const float *__restrict__ flags,
-                         int s_base, int s_end, int *__restrict__ status, long long budget, int no_loads)
+                         const float2 *__restrict__ ratio, const float *__restrict__ bandpass,
+                         const float2 *__restrict__ gains, int N, int S, int I_pad, int s_out, float scale,
+                         int rounds_per_cta, const float *__restrict__ flags, int s_base, int s_end,
+                         int *__restrict__ status, long long budget, int no_loads)
 {
     using W = Ws256;
-    constexpr int C = W::C, R = W::R, NF = W::NF, ROW = W::ROW, USZ = W::USZ, RS = W::RS, EJ = W::EJ, ESZ = W::ESZ;
+    constexpr int C = W::C, R = W::R, NF = W::NF, ROW = W::ROW, USZ = W::USZ, RS = W::RS, TW = W::TW, ESZ = W::ESZ;
     constexpr int ROW_BYTES = C * kPols * (int)sizeof(TIn);     // one raw time row of the station (both pols)
     constexpr int BUF_BYTES = kRound * ROW_BYTES;
-    constexpr int ALL = 2 * NF;
-    constexpr int NG = NF / 2;                  // FFT threads per group: group g takes rounds b = g mod 2
+    constexpr int NG = W::NG;
     constexpr int HAND = NF + NG;               // FULL / EMPTY: the FIR threads and one FFT group
     static_assert(OUT >= 2 && OUT <= 5, "planar outputs");
     static_assert(ROW_BYTES % 16 == 0, "rows must be whole 16-byte chunks");
     static_assert(ws256_smem_bytes<TIn>() <= 227 * 1024, "one CTA per SM");
 
     extern __shared__ __align__(16) unsigned char smem[];
-    float2 *tw = reinterpret_cast<float2 *>(smem);
-    unsigned char *inbuf = smem + C * sizeof(float2);
-    float2 *u = reinterpret_cast<float2 *>(inbuf + 2 * BUF_BYTES);   // [2][USZ]
-    float2 *et = u + 2 * USZ;                                         // [2][C][EJ]
-    float2 *bgt = et + 2 * ESZ;                                       // [C] bandpass x gain x scale
-    float2 *tw2 = bgt + C;                                            // [k1][n2] = W_C^(n2 k1): pass-1
-                                                                      // lanes (n2) read consecutive entries
-    const unsigned rbar = tc::smem_u32(tw2 + C);                      // raw-row mbarriers [2]
+    unsigned char *inbuf = smem;
+    float2 *u = reinterpret_cast<float2 *>(inbuf + 2 * BUF_BYTES);   // [NB][USZ]
+    float2 *et = u + W::NB * USZ;                                     // [NB][k1][spectrum] anchors
+    float2 *tw = et + W::NB * ESZ;                                        // [n2][TW] W_C^(n2 k1)
+    float2 *bpt = tw + R * TW;                                        // [k1][k2] bandpass of output k2, twice
+    const unsigned rbar = tc::smem_u32(bpt + C);                      // raw-row mbarriers [2]
     const int tid = threadIdx.x;
     const int sb = blockIdx.z;
     const int n = blockIdx.x / kPols, p = blockIdx.x % kPols;       // (station, pol) fastest
@@ -727,12 +754,11 @@ ppf_correct_ws256_kernel(const TIn *__restrict__ raw, void *__restrict__ corr, c
     const long long L = (long long)rows_total * C;
     const int nrounds = min(rounds_per_cta, (s_end - s0 + kRound - 1) / kRound);
 
-    for (int i = tid; i < C; i += ALL) {
-        tw[i] = twiddle[i];
-        tw2[i] = twiddle[(i % R) * (i / R)];
-        const float b = bandpass ? bandpass[(long long)n * C + i] : 1.f;
-        const float2 g = gains ? gains[n * kPols + p] : make_float2(1.f, 0.f);
-        bgt[i] = make_float2(b * g.x * scale, b * g.y * scale);
+    if (tid < C) {
+        const int hi = tid / R, lo = tid % R;
+        tw[hi * TW + lo] = twiddle[hi * lo];
+        const float bp = bandpass ? bandpass[(long long)n * C + hi + R * ((lo + R / 2) % R)] : 1.f;
+        bpt[tid] = make_float2(bp, bp);
     }
     if (tid == 0) {
         tc::mbar_init(rbar, 1);
@@ -755,11 +781,11 @@ ppf_correct_ws256_kernel(const TIn *__restrict__ raw, void *__restrict__ corr, c
             }
         };
         const int c = tid;
-        const float2 pst = phase[((long long)sb * N + n) * C + c];   // (phi0, step)
-        const float2 bgc = bgt[c];                                   // this input's bandpass x gain x scale
-        float sn1, cs1;
-        sincosf(pst.y, &sn1, &cs1);                                  // exp(i step)
-        const float2 rot = make_float2(cs1, sn1);
+        // anchor role: channel k1 + 128 (k1 = c / 16) of spectrum c % 16 of a round
+        const int aj = c % kRound;
+        const float2 pst = phase[((long long)sb * N + n) * C + C / 2 + c / kRound];   // (phi0, step)
+        const float2 gg = gains ? gains[n * kPols + p] : make_float2(1.f, 0.f);
+        const float2 gsc = make_float2(gg.x * scale, gg.y * scale);
         float2 h[T];
 #pragma unroll
         for (int k = 0; k < T; ++k) h[k] = make_float2(taps[k * C + c], taps[k * C + c]);
@@ -777,12 +803,28 @@ ppf_correct_ws256_kernel(const TIn *__restrict__ raw, void *__restrict__ corr, c
         if (nrounds > 1) issue(1, s0 + T - 1 + kRound, kRound);     // round 1: buffer 1, phase 1
 
         for (int b = 0; b < nrounds; ++b) {
-            const int q = b & 1;
+            const int q = b & 1, ub = b % W::NB;
             const int sr = s0 + b * kRound;
             raw_wait(rbar + 8u * q, (unsigned)(((b + q) / 2) & 1), status, budget);   // round b's rows
-            if (b >= 2) named_bar_sync(kBarEmpty + q, HAND);
+            // anchor of this round: phi reduced to [-pi, pi] (two-constant Cody-Waite
+            // split of 2 pi), __sincosf, times gain, scale and flag
+            float2 e;
+            {
+                const float phi = fmaf((float)(sr + aj), pst.y, pst.x);
+                const float kq = rintf(phi * 0.15915494309189535f);
+                float r = fmaf(-kq, 6.28125f, phi);
+                r = fmaf(-kq, 1.9353071795864769e-3f, r);
+                __sincosf(r, &e.y, &e.x);
+            }
+            e = cmul(gsc, e);
+            if (flags) {
+                const float fw = flags[(long long)n * S + min(sr + aj, S - 1)];
+                e = make_float2(e.x * fw, e.y * fw);
+            }
+            if (b >= W::NB) named_bar_sync(kBar256Empty + ub, HAND);
+            et[ub * ESZ + c] = e;
             const TIn *in = reinterpret_cast<const TIn *>(inbuf + q * BUF_BYTES);
-            float2 *uq = u + q * USZ;
+            float2 *uq = u + ub * USZ;
             // four outputs at a time (see the 16/64-channel kernel)
 #pragma unroll
             for (int j0 = 0; j0 < kRound; j0 += 4) {
@@ -804,128 +846,97 @@ ppf_correct_ws256_kernel(const TIn *__restrict__ raw, void *__restrict__ corr, c
                     win[(T - 1 + j0 + qq) % T] = t[qq];
                 }
             }
-            // phasors of this round: phi(sr) reduced to [-pi, pi] (two-constant
-            // Cody-Waite split of 2 pi) and __sincosf, then rotations by exp(i step)
-            float2 *eq = et + q * ESZ + c * EJ;
-            float2 e;
-            {
-                const float phi = fmaf((float)sr, pst.y, pst.x);
-                const float kq = rintf(phi * 0.15915494309189535f);
-                float r = fmaf(-kq, 6.28125f, phi);
-                r = fmaf(-kq, 1.9353071795864769e-3f, r);
-                __sincosf(r, &e.y, &e.x);
-            }
-            e = cmul(bgc, e);                           // the anchor carries bandpass x gain
-            if (flags) {
-#pragma unroll
-                for (int j = 0; j < kRound; ++j) {
-                    const float fw = flags[(long long)n * S + min(sr + j, S - 1)];
-                    eq[j] = make_float2(e.x * fw, e.y * fw);     // the whole per-sample factor
-                    e = cmul(e, rot);
-                }
-            } else {
-#pragma unroll
-                for (int j = 0; j < kRound; ++j) {
-                    eq[j] = e;
-                    e = cmul(e, rot);
-                }
-            }
-            named_bar_arrive(kBarFull + q, HAND);
+            named_bar_arrive(kBar256Full + ub, HAND);
             named_bar_sync(kBarRaw, NF);                // every FIR thread has read raw buffer q
             if (tid == 0) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             if (b + 2 < nrounds) issue(q, s0 + T - 1 + (b + 2) * kRound, kRound);
         }
     } else {
-        // ---------------- FFT threads: two groups of NG, group g = buffer g ----------------
+        // ---------------- FFT threads: group g takes rounds b = g mod 2 ----------------
         const int t = tid - NF;
         const int g = t / NG, tg = t % NG;
-        const int bar_fft = g ? kBarFft2 : kBarFft;
+        const int bar_fft = kBar256Fft + g;
         constexpr int planes = OUT == 4 ? 4 : 2;
         const long long pstride = (long long)I_pad * s_out;
         const int i = n * kPols + p;
+        const int S16 = (S + kRound - 1) / kRound * kRound;
+        // pass 1: column n2, rows tr0 and tr0 + 8; pass 2: k1, spectra jp and jp + 1
+        const int n2 = (tg % 32) / 2, tr0 = 2 * (tg / 32) + (tg & 1);
+        const int k1 = tg / 8, jp = 2 * (tg % 8);
         for (int b = g; b < nrounds; b += 2) {
-            const int q = b & 1;
+            const int q = b % W::NB;
             const int sr = s0 + b * kRound;
             float2 *uq = u + q * USZ;
-            const float2 *eq = et + q * ESZ;
-            named_bar_sync(kBarFull + q, HAND);
-            // pass 1: two (row tr = spectrum, column n2) tasks per thread
+            const float4 rr = *reinterpret_cast<const float4 *>(ratio + (long long)n * S16 + sr + jp);
+            named_bar_sync(kBar256Full + q, HAND);
             float2 v[2][R];
 #pragma unroll
-            for (int it = 0; it < 2; ++it) {
-                const int task = it * NG + tg;
-                const int tr = task / R, n2 = task % R;
+            for (int it = 0; it < 2; ++it)
 #pragma unroll
-                for (int n1 = 0; n1 < R; ++n1) v[it][n1] = uq[tr * ROW + R * n1 + n2];
-            }
+                for (int n1 = 0; n1 < R; ++n1) v[it][n1] = uq[(tr0 + 8 * it) * ROW + R * n1 + n2];
 #pragma unroll
-            for (int it = 0; it < 2; ++it) {
-                const int n2 = (it * NG + tg) % R;
-                fft_reg<R>(v[it]);
+            for (int it = 0; it < 2; ++it) fft_reg<R>(v[it]);
 #pragma unroll
-                for (int k1 = 1; k1 < R; ++k1) v[it][k1] = cmul(v[it][k1], tw2[k1 * R + n2]);
+            for (int kk = 0; kk < R; kk += 2) {
+                const float4 w = *reinterpret_cast<const float4 *>(tw + n2 * TW + kk);
+#pragma unroll
+                for (int it = 0; it < 2; ++it) {
+                    if (kk) v[it][kk] = cmul(v[it][kk], make_float2(w.x, w.y));
+                    v[it][kk + 1] = cmul(v[it][kk + 1], make_float2(w.z, w.w));
+                }
             }
             named_bar_sync(bar_fft, NG);                // every thread of the group has read u[q]
 #pragma unroll
-            for (int it = 0; it < 2; ++it) {
-                const int task = it * NG + tg;
-                const int tr = task / R, n2 = task % R;
+            for (int it = 0; it < 2; ++it)
 #pragma unroll
-                for (int k1 = 0; k1 < R; ++k1) uq[(k1 * R + n2) * RS + tr] = v[it][k1];
-            }
+                for (int kk = 0; kk < R; ++kk) uq[(kk * R + n2) * RS + tr0 + 8 * it] = v[it][kk];
             named_bar_sync(bar_fft, NG);                // P1 complete
-            // pass 2: two (k1, spectrum j) items per thread, a half-warp per k1
 #pragma unroll
-            for (int it = 0; it < 2; ++it) {
-                const int item = it * NG + tg;
-                const int k1 = item / 16, j = item % 16;
-#pragma unroll
-                for (int m = 0; m < R; ++m) v[it][m] = uq[(k1 * R + m) * RS + j];
+            for (int m = 0; m < R; ++m) {
+                const float4 w = *reinterpret_cast<const float4 *>(uq + (k1 * R + m) * RS + jp);
+                v[0][m] = make_float2(w.x, w.y);
+                v[1][m] = make_float2(w.z, w.w);
             }
+            const float4 ee = *reinterpret_cast<const float4 *>(et + q * ESZ + k1 * kRound + jp);
+            if (b + W::NB < nrounds) named_bar_arrive(kBar256Empty + q, HAND);
 #pragma unroll
-            for (int it = 0; it < 2; ++it) {
-                const int item = it * NG + tg;
-                const int k1 = item / 16, j = item % 16;
-                fft_reg<R>(v[it]);
+            for (int it = 0; it < 2; ++it) fft_reg<R>(v[it]);
+            // output k2 is channel k1 + 128 + 16 k2 for k2 < 8 and k1 + 128 + 16 (k2 - 16) above
+            float2 r[2] = {make_float2(rr.x, rr.y), make_float2(rr.z, rr.w)};
+            float2 up[2] = {make_float2(ee.x, ee.y), make_float2(ee.z, ee.w)}, dn[2];
 #pragma unroll
-                for (int k2 = 0; k2 < R; ++k2) {
-                    const int kout = k1 + R * ((k2 + R / 2) % R);
-                    v[it][k2] = cmul(v[it][k2], eq[kout * EJ + j]);
-                }
-            }
-            if (b + 2 < nrounds) named_bar_arrive(kBarEmpty + q, HAND);
+            for (int it = 0; it < 2; ++it) dn[it] = cmul(up[it], conj2(r[it]));
 #pragma unroll
-            for (int it = 0; it < 2; ++it) {
-                const int item = it * NG + tg;
-                const int k1 = item / 16, j = item % 16;
-                const int s = sr + j;
-                if (sr + kRound > s_end && s >= s_end) {       // only in the block's last round
+            for (int k2 = 0; k2 < R / 2; k2 += 2) {
+                const float4 bu = *reinterpret_cast<const float4 *>(bpt + k1 * R + k2);
+                const float4 bd = *reinterpret_cast<const float4 *>(bpt + k1 * R + R - 2 - k2);
+                const float2 fu[2] = {make_float2(bu.x, bu.y), make_float2(bu.z, bu.w)};
+                const float2 fd[2] = {make_float2(bd.z, bd.w), make_float2(bd.x, bd.y)};
 #pragma unroll
-                    for (int k2 = 0; k2 < R; ++k2) v[it][k2] = make_float2(0.f, 0.f);
-                }
-                const long long base = (long long)sb * C * planes * pstride + (long long)i * s_out + (s - s_base);
+                for (int qq = 0; qq < 2; ++qq) {
+                    const int ku = k2 + qq, kd = R - 1 - ku;
 #pragma unroll
-                for (int k2 = 0; k2 < R; ++k2) {
-                    const int kout = k1 + R * ((k2 + R / 2) % R);
-                    const float2 y = v[it][k2];
-                    const long long o = base + (long long)kout * planes * pstride;
-                    if constexpr (OUT == 5) {
-                        float *out = reinterpret_cast<float *>(corr);
-                        out[o] = y.x;
-                        out[o + pstride] = y.y;
-                    } else {
-                        unsigned short *out = reinterpret_cast<unsigned short *>(corr);
-                        const unsigned short hr = to_bits(y.x, OUT), hi = to_bits(y.y, OUT);
-                        out[o] = hr;
-                        out[o + pstride] = hi;
-                        if constexpr (OUT == 4) {
-                            out[o + 2 * pstride] =
-                                __half_as_ushort(__float2half_rn(y.x - __half2float(__ushort_as_half(hr))));
-                            out[o + 3 * pstride] =
-                                __half_as_ushort(__float2half_rn(y.y - __half2float(__ushort_as_half(hi))));
-                        }
+                    for (int it = 0; it < 2; ++it) {
+                        v[it][ku] = cmul(__fmul2_rn(v[it][ku], fu[qq]), up[it]);
+                        v[it][kd] = cmul(__fmul2_rn(v[it][kd], fd[qq]), dn[it]);
+                        up[it] = cmul(up[it], r[it]);
+                        dn[it] = cmul(dn[it], conj2(r[it]));
                     }
                 }
+            }
+            const int s = sr + jp;
+            if (sr + kRound > s_end) {                         // only in the block's last round
+#pragma unroll
+                for (int k2 = 0; k2 < R; ++k2) {
+                    if (s >= s_end) v[0][k2] = make_float2(0.f, 0.f);
+                    if (s + 1 >= s_end) v[1][k2] = make_float2(0.f, 0.f);
+                }
+            }
+            const long long base = (long long)sb * C * planes * pstride + (long long)i * s_out + (s - s_base);
+#pragma unroll
+            for (int k2 = 0; k2 < R; ++k2) {
+                const int kout = k1 + R * ((k2 + R / 2) % R);
+                store_planar<OUT>(corr, base + (long long)kout * planes * pstride, pstride, v[0][k2], v[1][k2]);
             }
         }
     }
@@ -992,8 +1003,8 @@ cudaError_t launch_t(const Handle &h, const void *raw, void *corr, const float *
         auto kern = ppf_correct_ws256_kernel<T, TIn, OUT>;
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        kern<<<grid, 2 * Ws256::NF, smem, st>>>(reinterpret_cast<const TIn *>(raw), corr, h.d_taps, h.d_twiddle,
-                                                h.d_phase, bandpass, gains, N, S, h.I_pad, s_out, scale, rpc, flags,
+        kern<<<grid, Ws256::ALL, smem, st>>>(reinterpret_cast<const TIn *>(raw), corr, h.d_taps, h.d_twiddle,
+                                                h.d_phase, h.d_ratio, bandpass, gains, N, S, h.I_pad, s_out, scale, rpc, flags,
                                                 s_base, s_end, h.d_status, h.tc_timeout_cycles,
                                                 h.tc_test_no_tma);
         e = cudaGetLastError();

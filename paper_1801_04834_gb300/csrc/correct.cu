@@ -29,16 +29,33 @@
 namespace fxi {
 namespace {
 
+// ratio (may be null): [N][S16] exp(2 pi i (fs / 16) tau_n(s)), the factor from a
+// channel of a 256-channel block to the sixteenth one on, rounded to FP32 only at
+// the end: the reduced angle's FP32 remainder turns the sine and cosine.
 __global__ void phase_table_kernel(const double *__restrict__ centres, const double *__restrict__ tau_b,
                                    const double *__restrict__ tau_e, float2 *__restrict__ table,
-                                   int SB, int N, int C, int S, double fs)
+                                   float2 *__restrict__ ratio, int SB, int N, int C, int S, double fs)
 {
+    const long long total = (long long)SB * N * C;
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long long)SB * N * C) return;
+    const double two_pi = 6.283185307179586476925286766559;
+    if (idx >= total) {
+        const int S16 = (S + 15) / 16 * 16;
+        const long long q = idx - total;
+        if (!ratio || q >= (long long)N * S16) return;
+        const int n = (int)(q / S16), s = (int)(q - (long long)n * S16);
+        const double tau = tau_b[n] + (tau_e[n] - tau_b[n]) * (double)s / (double)S;
+        const double cyc = fs / 16.0 * tau;
+        const double a = two_pi * (cyc - rint(cyc));
+        const float hi = (float)a, lo = (float)(a - (double)hi);
+        float sn, cs;
+        sincosf(hi, &sn, &cs);
+        ratio[q] = make_float2(fmaf(-sn, lo, cs), fmaf(cs, lo, sn));
+        return;
+    }
     const int k = (int)(idx % C);
     const int n = (int)((idx / C) % N);
     const int sb = (int)(idx / ((long long)C * N));
-    const double two_pi = 6.283185307179586476925286766559;
     const double f = centres[sb] + (double)(k - C / 2) * fs / (double)C;
     const double phi0 = two_pi * f * tau_b[n];
     const double red = phi0 - two_pi * rint(phi0 / two_pi);
@@ -274,11 +291,12 @@ static __device__ __align__(256) float2 g_noalloc_phase[FX_NOALLOC_MAX_PHASES];
 cudaError_t launch_phase_table(const Handle &h, const double *tau_b, const double *tau_e,
                                cudaStream_t st)
 {
-    const long long n = (long long)h.p.n_subbands * h.p.n_stations * h.p.n_channels;
+    const long long n = (long long)h.p.n_subbands * h.p.n_stations * h.p.n_channels +
+                        (h.d_ratio ? (long long)h.p.n_stations * ((h.p.n_spectra + 15) / 16 * 16) : 0);
     const int threads = 256;
     const long long blocks = (n + threads - 1) / threads;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    phase_table_kernel<<<(unsigned)blocks, threads, 0, st>>>(h.d_centres, tau_b, tau_e, h.d_phase,
+    phase_table_kernel<<<(unsigned)blocks, threads, 0, st>>>(h.d_centres, tau_b, tau_e, h.d_phase, h.d_ratio,
                                                              h.p.n_subbands, h.p.n_stations,
                                                              h.p.n_channels, h.p.n_spectra,
                                                              h.p.sample_rate_hz);
@@ -338,7 +356,7 @@ cudaError_t launch_correct_f32_noalloc(int N, int SB, int C, int S, double fs, c
     cudaError_t e = noalloc_phase_ptr(&table);
     if (e != cudaSuccess) return e;
     const long long n = (long long)SB * N * C;
-    phase_table_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(centres, tau_b, tau_e, table, SB, N, C, S,
+    phase_table_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(centres, tau_b, tau_e, table, nullptr, SB, N, C, S,
                                                                     fs);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;

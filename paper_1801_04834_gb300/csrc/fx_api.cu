@@ -170,6 +170,8 @@ extern "C" fx_status fx_create(const fx_params *pp, fx_handle **out)
     FX_TRY(cudaMalloc(&h->d_twiddle, sizeof(float2) * C));
     FX_TRY(cudaMalloc(&h->d_centres, sizeof(double) * SB));
     FX_TRY(cudaMalloc(&h->d_phase, sizeof(float2) * SB * N * C));
+    if (C == 256 && p.precision != FX_F32)
+        FX_TRY(cudaMalloc(&h->d_ratio, sizeof(float2) * N * (size_t)((S + 15) / 16 * 16)));
     FX_TRY(cudaMalloc(&h->d_status, sizeof(int) * 4));
     FX_TRY(cudaMalloc(&h->d_xf32_tiles, sizeof(int2) * ntiles));
     FX_TRY(cudaMalloc(&h->d_adj_partial, sizeof(double) * 4 * (size_t)fxi::adjoint_blocks(*h) * h->I));
@@ -209,6 +211,7 @@ extern "C" void fx_destroy(fx_handle *h)
     cudaFree(h->d_twiddle);
     cudaFree(h->d_centres);
     cudaFree(h->d_phase);
+    cudaFree(h->d_ratio);
     cudaFree(h->d_status);
     cudaFree(h->d_xf32_tiles);
     cudaFree(h->d_adj_partial);

@@ -82,7 +82,9 @@ enum {
     kBarFft = 2,     // FFT threads among themselves
     kBarFull = 3,    // FULL[0], FULL[1]: FIR round in the row buffer (ids 3, 4)
     kBarEmpty = 5,   // EMPTY[0], EMPTY[1]: FFT threads done with it (ids 5, 6)
-    kBarFft2 = 7,    // the second FFT group of the 256-channel kernel among itself
+    kBar256Full = 3,    // the 256-channel kernel's four row buffers: FULL (ids 3 to 6),
+    kBar256Empty = 7,   // EMPTY (ids 7 to 10)
+    kBar256Fft = 11,    // each of its two FFT groups among itself (ids 11, 12)
 };
 __device__ __forceinline__ void named_bar_sync(int id, int n)
 {
