@@ -534,10 +534,12 @@ extern "C" fx_status fx_correct_correlate_backward(fx_handle *h, const float *d_
 
 // The correlations inside the moving-delay adjoint: its FP64 gradients keep the
 // rounding of these two forms (xcorr_tf32.cu)
-static cudaError_t adjoint_xstage(const fx_handle &h, const void *corr, float2 *vis, cudaStream_t s)
+static cudaError_t adjoint_xstage(const fx_handle &h, void *corr, float2 *vis, bool weighted, cudaStream_t s)
 {
-    return h.p.precision == FX_F32 ? fxi::launch_xcorr_f32(h, static_cast<const float2 *>(corr), vis, s)
-                                   : fxi::launch_xcorr_tf32(h, static_cast<const float *>(corr), vis, s);
+    if (h.p.precision != FX_F32) return fxi::launch_xcorr_tf32(h, static_cast<const float *>(corr), vis, s, weighted);
+    cudaError_t e = weighted ? fxi::launch_weight_spectra(h, static_cast<float2 *>(corr), s) : cudaSuccess;
+    if (e == cudaSuccess) e = fxi::launch_xcorr_f32(h, static_cast<const float2 *>(corr), vis, s);
+    return e;
 }
 
 extern "C" fx_status fx_correct_correlate_backward_interp(
@@ -565,9 +567,8 @@ extern "C" fx_status fx_correct_correlate_backward_interp(
     cudaError_t e = fxi::launch_phase_table(*h, d_delay_begin, d_delay_end, s);
     if (e == cudaSuccess)   // the corrected block with unit gains: Y
         e = fxi::launch_correct(*h, reinterpret_cast<const float2 *>(d_chan), d_bandpass, nullptr, d_work_corr, s);
-    if (e == cudaSuccess) e = adjoint_xstage(*h, d_work_corr, K, s);                  // K = sum Y Y^H
-    if (e == cudaSuccess) e = fxi::launch_weight_spectra(*h, d_work_corr, s);         // Y sqrt(s/S)
-    if (e == cudaSuccess) e = adjoint_xstage(*h, d_work_corr, M1, s);                 // M1 = sum (s/S) Y Y^H
+    if (e == cudaSuccess) e = adjoint_xstage(*h, d_work_corr, K, false, s);           // K = sum Y Y^H
+    if (e == cudaSuccess) e = adjoint_xstage(*h, d_work_corr, M1, true, s);           // M1 = sum (s/S) Y Y^H
     if (e == cudaSuccess)
         e = fxi::launch_adjoint_interp(*h, K, M1, reinterpret_cast<const float2 *>(d_grad_vis),
                                        reinterpret_cast<const float2 *>(d_gains),

@@ -92,7 +92,7 @@ cudaError_t launch_apply_gains(const Handle &h, const float2 *R, const float2 *g
                                float2 *V, cudaStream_t st);
 cudaError_t launch_adjoint(const Handle &h, const float2 *R, const float2 *G, const float2 *gains,
                            const double *tau, float2 *grad_gains, double *grad_tau, cudaStream_t st);
-cudaError_t launch_weight_spectra(const Handle &h, void *corr, cudaStream_t st);
+cudaError_t launch_weight_spectra(const Handle &h, float2 *corr, cudaStream_t st);   // FX_F32 layout, in place
 cudaError_t launch_adjoint_interp(const Handle &h, const float2 *K, const float2 *M1, const float2 *G,
                                   const float2 *gains, float2 *grad_gains, double *grad_tb, double *grad_te,
                                   cudaStream_t st);
@@ -112,7 +112,8 @@ cudaError_t launch_xcorr_f32_tc(const Handle &h, const float2 *corr, float2 *vis
                                 bool accumulate = false);   // accumulate: add to vis
 
 // xcorr_tf32.cu (FX_TF32_SPLIT operands, every product formed: the moving-delay adjoint)
-cudaError_t launch_xcorr_tf32(const Handle &h, const float *corr, float2 *vis, cudaStream_t st);
+// weighted: spectrum s counts s / S (each operand times sqrt(s / S), rounded to FP32)
+cudaError_t launch_xcorr_tf32(const Handle &h, const float *corr, float2 *vis, cudaStream_t st, bool weighted);
 
 // probe.cu
 cudaError_t launch_ffma_probe(int iterations, int blocks, float *sink, cudaStream_t st);

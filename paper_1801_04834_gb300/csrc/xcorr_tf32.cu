@@ -127,6 +127,7 @@ struct T3Params {
     long long timeout_cycles;
     int ipc;                  // items per channel
     int N, nk, chunk;         // stations, stages per item, stages per accumulator chain
+    int S;                    // spectra of the block
     int stages;
     unsigned stage_bytes;
     unsigned a_off;           // byte offset of the B region when an A region precedes it
@@ -224,13 +225,26 @@ __device__ __forceinline__ uint2 neg_bf16x4(uint2 v) { return make_uint2(v.x ^ 0
 // the column operand (col) -hi R after the two TF32 planes and BF16 hi R,
 // hi J, -hi R, lo R, lo J, -lo R; for the row operand of an off-diagonal item
 // BF16 hi R, hi J, lo R, lo J.
+// W: the raw rows are first multiplied by the thread's four spectra's weights w
+// (the chunks a thread takes, t + 128 k, all hold the same four spectra).
+template <bool W>
 __device__ __forceinline__ void convert_split(unsigned char *tf, unsigned tf_pitch, unsigned char *bf,
-                                              unsigned bf_pitch, int rows, bool col, int t)
+                                              unsigned bf_pitch, int rows, bool col, int t, float4 w)
 {
     const int nq = rows * (int)(kT3RowBytes / 16);
     for (int q = t; q < nq; q += 128) {
-        const uint4 x = reinterpret_cast<const uint4 *>(tf)[q];
-        const uint4 y = reinterpret_cast<const uint4 *>(tf + tf_pitch)[q];
+        uint4 x = reinterpret_cast<const uint4 *>(tf)[q];
+        uint4 y = reinterpret_cast<const uint4 *>(tf + tf_pitch)[q];
+        if constexpr (W) {
+            auto mul = [&](uint4 v) {
+                return make_uint4(__float_as_uint(__uint_as_float(v.x) * w.x), __float_as_uint(__uint_as_float(v.y) * w.y),
+                                  __float_as_uint(__uint_as_float(v.z) * w.z), __float_as_uint(__uint_as_float(v.w) * w.w));
+            };
+            x = mul(x);
+            y = mul(y);
+            reinterpret_cast<uint4 *>(tf)[q] = x;
+            reinterpret_cast<uint4 *>(tf + tf_pitch)[q] = y;
+        }
         uint4 xh, xl, yh, yl;
         xh.x = hi_bits(x.x); xh.y = hi_bits(x.y); xh.z = hi_bits(x.z); xh.w = hi_bits(x.w);
         yh.x = hi_bits(y.x); yh.y = hi_bits(y.y); yh.z = hi_bits(y.z); yh.w = hi_bits(y.w);
@@ -256,6 +270,7 @@ __device__ __forceinline__ void convert_split(unsigned char *tf, unsigned tf_pit
     }
 }
 
+template <bool W>
 __global__ void __launch_bounds__(kT3Threads, 1) xcorr_tf32_kernel(const __grid_constant__ T3Params P)
 {
     extern __shared__ unsigned char smem_raw[];
@@ -431,9 +446,17 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_tf32_kernel(const __grid_
                 }
                 unsigned char *st = tiles + (size_t)s * P.stage_bytes;
                 unsigned char *bb = diag ? st : st + P.a_off;
+                float4 w = make_float4(1.f, 1.f, 1.f, 1.f);
+                if constexpr (W) {                       // sqrt(s / S): lane l works out spectrum l mod 16
+                    const int s1 = kc * kT3K + (lane & 15);
+                    const float mine = s1 < P.S ? sqrtf((float)s1 / (float)P.S) : 0.f;
+                    const int s4 = 4 * ((ct & 3) ^ ((ct >> 3) & 3));      // this thread's chunks: spectra s4 .. s4 + 3
+                    w = make_float4(__shfl_sync(0xffffffffu, mine, s4), __shfl_sync(0xffffffffu, mine, s4 + 1),
+                                    __shfl_sync(0xffffffffu, mine, s4 + 2), __shfl_sync(0xffffffffu, mine, s4 + 3));
+                }
                 if (!diag)   // row inputs: BF16 planes after the two TF32 planes of the A region
-                    convert_split(st, kT3APlane, st + kT3ABf, kT3ABfPlane, 128, false, ct);
-                convert_split(bb, pitch, bb + 3 * pitch, (unsigned)n * kT3BfRowBytes, n, true, ct);
+                    convert_split<W>(st, kT3APlane, st + kT3ABf, kT3ABfPlane, 128, false, ct, w);
+                convert_split<W>(bb, pitch, bb + 3 * pitch, (unsigned)n * kT3BfRowBytes, n, true, ct, w);
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
                 if (lane == 0) mbar_arrive(conv_bar(s));
@@ -561,7 +584,7 @@ bool t3_plan(int I_pad, int NT, T3Plan &pl)
 
 }  // namespace
 
-cudaError_t launch_xcorr_tf32(const Handle &h, const float *corr, float2 *vis, cudaStream_t st)
+cudaError_t launch_xcorr_tf32(const Handle &h, const float *corr, float2 *vis, cudaStream_t st, bool weighted)
 {
     EncodeTiledFn enc = t3_encode_fn();
     if (!enc) return cudaErrorNotSupported;
@@ -593,6 +616,7 @@ cudaError_t launch_xcorr_tf32(const Handle &h, const float *corr, float2 *vis, c
     P.n_items = planes / 2 * P.ipc;
     P.N = h.p.n_stations;
     P.nk = h.S_pad / kT3K;
+    P.S = h.p.n_spectra;
     P.chunk = chunk;
     P.B = h.B;
     P.stages = pl.stages;
@@ -601,11 +625,12 @@ cudaError_t launch_xcorr_tf32(const Handle &h, const float *corr, float2 *vis, c
     P.timeout_cycles = h.tc_timeout_cycles;
     P.no_tma = h.tc_test_no_tma;
     const size_t smem = 1024 + (size_t)pl.stages * pl.stage_bytes + 8 * kT3Bars + 16;
-    cudaError_t e = cudaFuncSetAttribute(xcorr_tf32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    auto kern = weighted ? xcorr_tf32_kernel<true> : xcorr_tf32_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const long long grid = std::min<long long>(P.n_items, h.num_sms);
     if (grid <= 0) return cudaSuccess;
-    xcorr_tf32_kernel<<<(unsigned)grid, kT3Threads, smem, st>>>(P);
+    kern<<<(unsigned)grid, kT3Threads, smem, st>>>(P);
     return cudaGetLastError();
 }
 
