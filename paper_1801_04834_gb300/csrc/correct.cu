@@ -230,6 +230,23 @@ correct_planar_kernel(const float2 *__restrict__ chan, const float2 *__restrict_
     __syncthreads();
     constexpr int planes = (MODE == 3) ? 4 : 2;
     const long long plane_stride = (long long)I_pad * S_pad;
+    if constexpr (MODE == 4) {
+        // task = (pol p, channel c, group of 4 spectra): eight lanes of a store fill a
+        // 128-byte run (groups of 8 left every other 16 bytes to a second store)
+        for (int task = threadIdx.x; task < kPols * CC * (ST / 4); task += kNT) {
+            const int g4 = task % (ST / 4);
+            const int c = (task / (ST / 4)) % CC;
+            const int p = task / ((ST / 4) * CC);
+            const int sg = s0 + g4 * 4;
+            if (sg >= S_pad) continue;
+            const float2 *src = tile + (p * CC + c) * TR + g4 * 4;
+            float *out = reinterpret_cast<float *>(corr) + (((long long)sb * C + c0 + c) * planes) * plane_stride +
+                         (long long)(n * kPols + p) * S_pad + sg;
+            *reinterpret_cast<float4 *>(out) = make_float4(src[0].x, src[1].x, src[2].x, src[3].x);
+            *reinterpret_cast<float4 *>(out + plane_stride) = make_float4(src[0].y, src[1].y, src[2].y, src[3].y);
+        }
+        return;
+    }
     // task = (pol p, channel c, group of 8 spectra)
     for (int task = threadIdx.x; task < kPols * CC * (ST / 8); task += kNT) {
         const int g8 = task % (ST / 8);
@@ -240,14 +257,7 @@ correct_planar_kernel(const float2 *__restrict__ chan, const float2 *__restrict_
         const float2 *src = tile + (p * CC + c) * TR + g8 * 8;
         const long long base = (((long long)sb * C + c0 + c) * planes) * plane_stride +
                                (long long)(n * kPols + p) * S_pad + sg;
-        if constexpr (MODE == 4) {
-            float4 *re = reinterpret_cast<float4 *>(reinterpret_cast<float *>(corr) + base);
-            float4 *im = reinterpret_cast<float4 *>(reinterpret_cast<float *>(corr) + base + plane_stride);
-            re[0] = make_float4(src[0].x, src[1].x, src[2].x, src[3].x);
-            re[1] = make_float4(src[4].x, src[5].x, src[6].x, src[7].x);
-            im[0] = make_float4(src[0].y, src[1].y, src[2].y, src[3].y);
-            im[1] = make_float4(src[4].y, src[5].y, src[6].y, src[7].y);
-        } else {
+        if constexpr (MODE != 4) {
             unsigned short re_hi[8], im_hi[8], re_lo[8], im_lo[8];
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
