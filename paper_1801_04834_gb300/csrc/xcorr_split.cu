@@ -127,6 +127,7 @@ constexpr int kT3AccCols = 256;
 constexpr int kT3Bars = 4 * kT3MaxStages + 6;         // full, conv, empty, landed per stage; accf 2, acce 2, exch, drain
 constexpr int kT3Blk = 32 * 33;                       // one 32 x 32 block of the transpose scratch, padded rows
 constexpr unsigned kT3Scratch = 10u * kT3Blk * 4u;    // lower block triangle of a 128 x 128 plane
+constexpr unsigned kT3ScratchSmall = 4u * kT3Blk * 4u; // four blocks at a time
 constexpr unsigned kT3SmemMax = 227u * 1024u;
 
 struct T3Params {
@@ -140,7 +141,9 @@ struct T3Params {
     long long n_items;        // ceil(SB * C / group) * ipc
     long long channels;       // SB * C
     int group;                // channels per item: > 1 only with one diagonal item per channel
-    int gin;                  // inputs (padded) per channel of a group
+    int segs;                 // time segments of one channel side by side in a tile (then group = 1)
+    int gin;                  // inputs (padded) per channel or segment of a tile
+    int nk_all;               // stages of a channel: nk per segment
     long long B;              // baselines
     long long timeout_cycles;
     int ipc;                  // items per channel
@@ -148,6 +151,8 @@ struct T3Params {
     int nr;                   // rows of mapr's box
     int stages, lands;        // depth of the operand ring and of the landing ring
     unsigned stage_bytes, land_bytes;
+    unsigned row_land;        // blocked: offset of the row inputs' stations in a landing slot
+    unsigned scratch_bytes;   // kT3Scratch or kT3ScratchSmall
     int no_tma;               // failure-detection test hook: issue no loads
     int accumulate;           // add to vis
 };
@@ -328,14 +333,14 @@ __device__ __forceinline__ void convert_planar(unsigned char *tf, unsigned tp, u
 // Spectrum-blocked operands: `land` holds stations' runs of [16 spectra][2
 // pols] complex values; a task is 4 spectra of one station, both pols, written
 // to the TF32 planes (64-byte rows, 64-byte swizzle, pitch tp) too. Spectra from
-// s_lim on count as zero. The four 16-byte reads of a task are rotated by
+// s_lim on count as zero (every gst stations seg fewer: time segments). The four 16-byte reads of a task are rotated by
 // lane / 2 so that eight lanes' reads fall on distinct banks, and sorted again
 // in registers. Rows are ordered pol by pol within eight stations (row 16 (st /
 // 8) + 8 p + st mod 8), so that the lanes of a store take consecutive rows and
 // distinct banks too.
-template <int ROLE>
+template <int ROLE, bool SEG>
 __device__ __forceinline__ void convert_blocked(const unsigned char *land, unsigned char *tf, unsigned tp,
-                                                unsigned char *bf, unsigned bp, int rows, int s_lim, int t)
+                                                unsigned char *bf, unsigned bp, int rows, int s_lim, int gst, int seg, int t)
 {
     const int nt = rows / 2 * 4;                          // a multiple of 32: whole warps
     const int rot = (t >> 1) & 3;
@@ -349,10 +354,11 @@ __device__ __forceinline__ void convert_blocked(const unsigned char *land, unsig
 #pragma unroll
         for (int e = 0; e < 4; ++e) v[e] = rot & 2 ? u[(e + 2) & 3] : u[e];
         const int lc = q & 3, st = q >> 2;
-        if (s_lim < kT3K) {
+        const int lim = SEG ? s_lim - st / gst * seg : s_lim;
+        if (lim < kT3K) {
 #pragma unroll
             for (int e = 0; e < 4; ++e)
-                if (4 * lc + e >= s_lim) v[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (4 * lc + e >= lim) v[e] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
         float top = 0.f;
 #pragma unroll
@@ -381,7 +387,8 @@ __device__ __forceinline__ void convert_blocked(const unsigned char *land, unsig
 }
 
 // BLOCKED: spectrum-blocked complex operands (FX_F32), else planar (FX_TF32_SPLIT)
-template <bool BLOCKED>
+// (SEG: time segments of one channel share a tile)
+template <bool BLOCKED, bool SEG>
 __global__ void __launch_bounds__(kT3Threads, 1) xcorr_split_kernel(const __grid_constant__ T3Params P)
 {
     extern __shared__ unsigned char smem_raw[];
@@ -392,7 +399,7 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_split_kernel(const __grid
     unsigned char *land = tiles + (size_t)P.stages * P.stage_bytes;
     const unsigned land_u32 = tiles_u32 + (unsigned)P.stages * P.stage_bytes;
     float *scratch = reinterpret_cast<float *>(land + (size_t)P.lands * P.land_bytes);
-    unsigned char *ctrl = reinterpret_cast<unsigned char *>(scratch) + kT3Scratch;
+    unsigned char *ctrl = reinterpret_cast<unsigned char *>(scratch) + P.scratch_bytes;
     const unsigned bar0 = smem_u32(ctrl);
     auto full_bar = [&](int s) { return bar0 + 8u * s; };                          // rows landed
     auto conv_bar = [&](int s) { return bar0 + 8u * (kT3MaxStages + s); };         // operands written
@@ -461,7 +468,7 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_split_kernel(const __grid
                     const unsigned bbytes = (unsigned)min(n / 2, P.N - bst) * kT3StRun;
                     const unsigned tx = BLOCKED ? (diag ? 0u : abytes) + (P.group > 1 ? chans * P.N * kT3StRun : bbytes)
                                                 : (diag ? 0u : 2u * TA) + 2u * pitch;
-                    const long long chstep = P.nk * P.N * (long long)kT3StRun;
+                    const long long chstep = P.nk_all * P.N * (long long)kT3StRun;
                     const unsigned char *src = P.blk + gch * P.group * chstep;
                     for (int kc = 0; kc < slots; ++kc, ring.step(P.lands)) {
                         const int l = ring.i;
@@ -471,6 +478,17 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_split_kernel(const __grid
                         }
                         if (P.no_tma) continue;
                         filled = min(filled + 1, P.lands);
+                        if constexpr (BLOCKED && SEG) {
+                            // block kc of every segment (none past the channel's end: the
+                            // converter counts those spectra as zero)
+                            const unsigned run = (unsigned)P.N * kT3StRun;
+                            const int live = (P.nk_all - kc + P.nk - 1) / P.nk;
+                            mbar_arrive_expect_tx(full_bar(l), live * run);
+                            for (int c = 0; c < live; ++c)
+                                bulk_g2s(land_u32 + (unsigned)l * P.land_bytes + (unsigned)(c * (P.gin / 2)) * kT3StRun,
+                                         src + (long long)(kc + c * P.nk) * run, run, full_bar(l));
+                            continue;
+                        }
                         mbar_arrive_expect_tx(full_bar(l), tx);
                         const unsigned dst = land_u32 + (unsigned)l * P.land_bytes;
                         if constexpr (BLOCKED) {
@@ -482,10 +500,16 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_split_kernel(const __grid
                                 continue;
                             }
                             bulk_g2s(dst, b + (long long)bst * kT3StRun, bbytes, full_bar(l));
-                            if (!diag) bulk_g2s(dst + 64u * kT3StRun, b + (long long)ast * kT3StRun, abytes, full_bar(l));
+                            if (!diag) bulk_g2s(dst + P.row_land, b + (long long)ast * kT3StRun, abytes, full_bar(l));
                         } else {
                             for (int pl = 0; pl < 2; ++pl) {
                                 const int z = (int)(gch * P.group * 2 + pl), x = kc * 2 * kT3K;
+                                if constexpr (SEG) {   // spectra past the padded end arrive as zeros
+                                    for (int c = 0; c < P.segs; ++c)
+                                        tma_load_3d(dst + (unsigned)pl * pitch + (unsigned)(c * P.gin) * TROW, &P.mapr,
+                                                    full_bar(l), x + c * P.nk * kT3K, 0, z);
+                                    continue;
+                                }
                                 if (P.group > 1) {     // channels past the last one arrive as zeros
                                     for (int c = 0; c < P.group; ++c)
                                         tma_load_3d(dst + (unsigned)pl * pitch + (unsigned)(c * P.gin) * TROW, &P.mapr,
@@ -632,13 +656,13 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_split_kernel(const __grid
                     unsigned char *st = tiles + (size_t)s * P.stage_bytes;
                     unsigned char *la = land + (size_t)l * P.land_bytes;
                     if constexpr (BLOCKED) {
-                        const int lim = P.S - kc * kT3K;
+                        const int lim = P.S - kc * kT3K, gst = P.gin / 2, seg = P.nk * kT3K;
                         if (diag) {
-                            convert_blocked<DIAG>(la, st, pitch, st + 2 * pitch, bpitch, n, lim, ct);
+                            convert_blocked<DIAG, SEG>(la, st, pitch, st + 2 * pitch, bpitch, n, lim, gst, seg, ct);
                         } else {
                             unsigned char *tb = st + 2 * TA + 4 * kT3ABf;
-                            convert_blocked<ROWS>(la + 64 * kT3StRun, st, TA, st + 2 * TA, kT3ABf, 128, lim, ct);
-                            convert_blocked<COLS>(la, tb + pitch, pitch, tb + 3 * pitch, bpitch, n, lim, ct);
+                            convert_blocked<ROWS, false>(la + P.row_land, st, TA, st + 2 * TA, kT3ABf, 128, lim, gst, seg, ct);
+                            convert_blocked<COLS, false>(la, tb + pitch, pitch, tb + 3 * pitch, bpitch, n, lim, gst, seg, ct);
                         }
                     } else {
                         const int half = kc % PER;
@@ -670,7 +694,7 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_split_kernel(const __grid
             const long long gch = w / P.ipc;
             const int row0 = itm.x, col0 = itm.y, n = itm.z;
             const bool diag = itm.w != 0;
-            const bool act = row0 + 32 * qd < (P.group > 1 ? n : 2 * P.N);   // some of this warp's rows are inputs
+            const bool act = row0 + 32 * qd < ((SEG || P.group > 1) ? n : 2 * P.N);   // some of this warp's rows are inputs
             float2 Q[32], V[32];                         // column pairs, for packed adds
 #pragma unroll
             for (int k = 0; k < 32; ++k) Q[k] = V[k] = make_float2(0.f, 0.f);
@@ -704,23 +728,36 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_split_kernel(const __grid
                 if (lane == 0) mbar_arrive(acce_bar(ab));
             }
             if (!live) break;
+            auto sync8 = [&]() {
+                __syncwarp();
+                if (lane == 0) mbar_arrive(exch_bar);
+                const bool got = t3wait(exch_bar, exch_it & 1u, abort_flag, P, 3);
+                ++exch_it;
+                return __all_sync(0xffffffffu, got) != 0;
+            };
             if (diag) {
                 // Re V = (P + P') / 2, Im V = Q - Q': each warp puts its 32 x 32 blocks
                 // on or below the diagonal into the scratch and reads the mirror
-                // blocks of those on or above it (rows of 33 words: no bank conflicts)
-                auto sync8 = [&]() {
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(exch_bar);
-                    const bool got = t3wait(exch_bar, exch_it & 1u, abort_flag, P, 3);
-                    ++exch_it;
-                    return __all_sync(0xffffffffu, got) != 0;
+                // blocks of those on or above it (rows of 33 words: no bank
+                // conflicts), all ten blocks at once or, with the small scratch, in
+                // three phases of three, three and the four diagonal ones
+                const bool small = P.scratch_bytes < kT3Scratch;
+                auto place = [&](int r, int c, int &slot) {     // block (r, c), c <= r: phase and slot
+                    if (!small) {
+                        slot = r * (r + 1) / 2 + c;
+                        return 0;
+                    }
+                    const int o = r * (r - 1) / 2 + c;
+                    slot = r == c ? r : o % 3;
+                    return r == c ? 2 : o / 3;
                 };
-                auto put = [&](const float2 (&A)[32]) {
+                auto put = [&](const float2 (&A)[32], int phase) {
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         const int cb = 2 * g + h;
-                        if (act && cb <= qd && 32 * cb < n) {
-                            float *s = scratch + (qd * (qd + 1) / 2 + cb) * kT3Blk + lane * 33;
+                        int slot;
+                        if (act && cb <= qd && 32 * cb < n && place(qd, cb, slot) == phase) {
+                            float *s = scratch + slot * kT3Blk + lane * 33;
 #pragma unroll
                             for (int j = 0; j < 16; ++j) {
                                 s[2 * j] = A[16 * h + j].x;
@@ -729,12 +766,13 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_split_kernel(const __grid
                         }
                     }
                 };
-                auto take = [&](float2 (&A)[32], float keep, float other) {
+                auto take = [&](float2 (&A)[32], int phase, float keep, float other) {
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         const int cb = 2 * g + h;
-                        if (act && cb >= qd && 32 * cb < n) {
-                            const float *s = scratch + (cb * (cb + 1) / 2 + qd) * kT3Blk + lane;
+                        int slot;
+                        if (act && cb >= qd && 32 * cb < n && place(cb, qd, slot) == phase) {
+                            const float *s = scratch + slot * kT3Blk + lane;
 #pragma unroll
                             for (int j = 0; j < 16; ++j) {
                                 float2 &v = A[16 * h + j];
@@ -744,17 +782,20 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_split_kernel(const __grid
                         }
                     }
                 };
-                put(V);
-                live = sync8();
-                if (!live) break;
-                take(V, 0.5f, 0.5f);
-                live = sync8();
-                if (!live) break;
-                put(Q);
-                live = sync8();
-                if (!live) break;
-                take(Q, 1.f, -1.f);
-                live = sync8();
+                for (int ph = 0; ph < (small ? 3 : 1) && live; ++ph) {
+                    put(V, ph);
+                    live = sync8();
+                    if (!live) break;
+                    take(V, ph, 0.5f, 0.5f);
+                    live = sync8();
+                }
+                for (int ph = 0; ph < (small ? 3 : 1) && live; ++ph) {
+                    put(Q, ph);
+                    live = sync8();
+                    if (!live) break;
+                    take(Q, ph, 1.f, -1.f);
+                    live = sync8();
+                }
                 if (!live) break;
             }
             // this lane's row input (blocked: rows pol by pol within eight stations, as
@@ -762,11 +803,45 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_split_kernel(const __grid
             constexpr int QN = BLOCKED ? 8 : 1;
             const int slot = (row0 >> 1) + 16 * qd + (BLOCKED ? 8 * (lane >> 4) + (lane & 7) : lane >> 1);
             const int p = BLOCKED ? (lane >> 3) & 1 : lane & 1;
-            // a group's channels take P.gin / 2 station slots each
-            const int cg = P.group > 1 ? slot / (P.gin >> 1) : 0;
+            // a group's channels (or segments) take P.gin / 2 station slots each
+            const int cg = (SEG || P.group > 1) ? slot / (P.gin >> 1) : 0;
             const int first = cg * (P.gin >> 1), i = slot - first;
             const long long ch = gch * P.group + cg;
             const bool mine = act && cg < P.group && ch < P.channels;
+            if constexpr (SEG) {
+                // the segments' diagonal blocks through the scratch (planes Re, Im of segs x
+                // gin x gin), then each entry's sum over the segments in their order
+                const int area = P.gin * P.gin, plane = P.segs * area;
+                const int row = 32 * qd + lane - cg * P.gin, from = cg * P.gin - 64 * g;
+                if (act && cg < P.segs) {
+                    float *s = scratch + cg * area + row * P.gin - from;
+#pragma unroll
+                    for (int k = 0; k < 64; ++k)
+                        if ((unsigned)(k - from) < (unsigned)P.gin) {
+                            s[k] = k & 1 ? V[k / 2].y : V[k / 2].x;
+                            s[plane + k] = k & 1 ? Q[k / 2].y : Q[k / 2].x;
+                        }
+                }
+                live = sync8();
+                if (!live) break;
+                for (int e = threadIdx.x; e < area; e += 32 * kT3EpiWarps) {
+                    const int a = e / P.gin, b = e - a * P.gin;
+                    const int ei = BLOCKED ? 8 * (a >> 4) + (a & 7) : a >> 1, ep = BLOCKED ? (a >> 3) & 1 : a & 1;
+                    const int ej = BLOCKED ? 8 * (b >> 4) + (b & 7) : b >> 1, eq = BLOCKED ? (b >> 3) & 1 : b & 1;
+                    if (ei > ej || ej >= P.N) continue;
+                    float2 v = make_float2(0.f, 0.f);
+                    for (int c = 0; c < P.segs; ++c) {
+                        v.x += scratch[c * area + e];
+                        v.y += scratch[plane + c * area + e];
+                    }
+                    float2 *dst = P.vis + (gch * P.B + (long long)ej * (ej + 1) / 2 + ei) * 4 + 2 * ep + eq;
+                    if (P.accumulate) v = make_float2(v.x + dst->x, v.y + dst->y);
+                    *dst = v;
+                }
+                live = sync8();
+                if (!live) break;
+                continue;
+            }
             float2 *vrow = P.vis + ch * P.B * 4 + (long long)i * 4 + 2 * p;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -829,22 +904,34 @@ int t3_group(int I_pad, long long channels, int num_sms)
     return (int)std::max<long long>(1, std::min<long long>(128 / I_pad, channels / num_sms));
 }
 
+// Time segments per item where there are not even two channels per SM to group: up
+// to 24 stations (48 inputs), a channel's spectra in 128 / I_pad segments side by
+// side, at least four stages each, whose diagonal blocks are summed at the end (8
+// stations x 64 channels x 768 spectra: 29 us in one, 16 us in eight). More stations leave
+// no room in the tile, or in the scratch for the blocks.
+int t3_segments(int I_pad, int group, int nk)
+{
+    static_assert(2u * 2u * 48u * 48u * 4u <= kT3Scratch && 2u * 4u * 32u * 32u * 4u <= kT3Scratch,
+                  "the segments' blocks fit the scratch");
+    return group > 1 || I_pad > 48 ? 1 : std::max(1, std::min(128 / I_pad, nk / 4));
+}
+
 // Item list of one channel (or group) and the shared-memory geometry it needs.
 struct T3Plan {
     std::vector<int4> items;
-    unsigned stage_bytes = 0, land_bytes = 0;
+    unsigned stage_bytes = 0, land_bytes = 0, row_land = 0, scratch_bytes = 0;
     int stages = 0, lands = 0;
 };
 
-bool t3_plan(int I_pad, bool blocked, int group, T3Plan &pl)
+bool t3_plan(int I_pad, bool blocked, int side, T3Plan &pl)
 {
     constexpr int NT = 64;                              // columns of an off-diagonal item
     pl.items.clear();
-    bool off = false;
+    unsigned nmax = 0;                                  // widest off-diagonal item
     const unsigned trow = blocked ? 64u : 128u;         // bytes of a TF32 row; planar: in the landing slot
     unsigned tf = 0, bf = 0;
     for (int row0 = 0; row0 < I_pad; row0 += 128) {
-        const unsigned nd = (unsigned)std::min(128, I_pad - row0) * group;
+        const unsigned nd = (unsigned)std::min(128, I_pad - row0) * side;
         pl.items.push_back(make_int4(row0, row0, (int)nd, 1));
         // the planes, and the 128-row reads of the A operands J (TF32) and hJ (BF16)
         tf = std::max(tf, std::max(2u * nd, nd + 128u) * trow);
@@ -852,7 +939,7 @@ bool t3_plan(int I_pad, bool blocked, int group, T3Plan &pl)
         for (int c0 = row0 + 128; c0 < I_pad; c0 += NT) {
             const int n = std::min(NT, I_pad - c0);
             pl.items.push_back(make_int4(row0, c0, n, 0));
-            off = true;
+            nmax = std::max(nmax, (unsigned)n);
             tf = std::max(tf, (256u + 3u * n) * trow);
             bf = std::max(bf, (512u + 6u * n) * kT3BfRow);
         }
@@ -862,8 +949,12 @@ bool t3_plan(int I_pad, bool blocked, int group, T3Plan &pl)
     // planes, so a diagonal item's need is below the sum too)
     const unsigned k1 = 1023u;
     pl.stage_bytes = ((blocked ? tf + bf : bf) + k1) & ~k1;
-    pl.land_bytes = ((blocked ? 64u * kT3StRun * (off ? 2u : 1u) : tf) + k1) & ~k1;
-    const unsigned room = kT3SmemMax - 1024u - kT3Scratch - 8u * kT3Bars - 16u;
+    pl.land_bytes = ((blocked ? (64u + nmax / 2) * kT3StRun : tf) + k1) & ~k1;
+    pl.row_land = nmax / 2 * kT3StRun;
+    // off-diagonal items have larger stages: the small scratch makes room for a third
+    // of them up to 80 stations (78 stations x 1024 channels x 1001 spectra: 873 -> 779 us)
+    pl.scratch_bytes = nmax ? kT3ScratchSmall : kT3Scratch;
+    const unsigned room = kT3SmemMax - 1024u - pl.scratch_bytes - 8u * kT3Bars - 16u;
     pl.stages = std::min<int>(kT3MaxStages - 1, (int)(room / (pl.stage_bytes + pl.land_bytes)));
     // blocked slots hold one stage: one more of them where it fits
     pl.lands = pl.stages + (blocked && (pl.stages + 1) * pl.land_bytes + pl.stages * pl.stage_bytes <= room ? 1 : 0);
@@ -876,7 +967,9 @@ cudaError_t t3_launch(const Handle &h, const void *corr, float2 *vis, cudaStream
     T3Plan pl;
     const long long channels = (long long)h.p.n_subbands * h.p.n_channels;
     const int group = t3_group(h.I_pad, channels, h.num_sms);
-    if (!t3_plan(h.I_pad, BLOCKED, group, pl)) return cudaErrorNotSupported;
+    const int nk = (h.p.n_spectra + kT3K - 1) / kT3K;
+    const int segs = t3_segments(h.I_pad, group, nk);
+    if (!t3_plan(h.I_pad, BLOCKED, group * segs, pl)) return cudaErrorNotSupported;
     if (2 * channels > 0x7fffffffLL) return cudaErrorInvalidValue;
     T3Params P;
     memset(&P, 0, sizeof(P));
@@ -909,19 +1002,24 @@ cudaError_t t3_launch(const Handle &h, const void *corr, float2 *vis, cudaStream
     P.n_items = (channels + group - 1) / group * P.ipc;
     P.N = h.p.n_stations;
     P.S = h.p.n_spectra;
-    P.nk = (h.p.n_spectra + kT3K - 1) / kT3K;
+    P.segs = segs;
+    P.nk_all = nk;
+    P.nk = (nk + segs - 1) / segs;
+    if (!BLOCKED && segs > 1) P.nk = (P.nk + 1) / 2 * 2;   // landing slots hold two stages
     P.chunk = chunk;
     P.B = h.B;
     P.stages = pl.stages;
     P.lands = pl.lands;
     P.stage_bytes = pl.stage_bytes;
     P.land_bytes = pl.land_bytes;
+    P.row_land = pl.row_land;
+    P.scratch_bytes = pl.scratch_bytes;
     P.timeout_cycles = h.tc_timeout_cycles;
     P.no_tma = h.tc_test_no_tma;
     P.accumulate = accumulate ? 1 : 0;
-    const size_t smem = 1024 + (size_t)pl.stages * pl.stage_bytes + (size_t)pl.lands * pl.land_bytes + kT3Scratch +
+    const size_t smem = 1024 + (size_t)pl.stages * pl.stage_bytes + (size_t)pl.lands * pl.land_bytes + pl.scratch_bytes +
                         8 * kT3Bars + 16;
-    auto kern = xcorr_split_kernel<BLOCKED>;
+    auto kern = segs > 1 ? xcorr_split_kernel<BLOCKED, true> : xcorr_split_kernel<BLOCKED, false>;
     // the register split draws on what the launch brings: refuse a build with less
     cudaFuncAttributes fa;
     cudaError_t e = cudaFuncGetAttributes(&fa, kern);

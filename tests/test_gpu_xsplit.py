@@ -1,6 +1,6 @@
 """X-stages on the tensor cores with FP32 operands (FX_TF32_SPLIT and, from 128
 spectra on, FX_F32) on given operands against an FP64 product: small arrays
-whose channels share a tile, ragged row blocks, integrations that end inside a
+whose channels, or time segments, share a tile, ragged row blocks, integrations that end inside a
 16-spectrum block, every accumulator chain length of FX_F32.
 
 Bound: a real accumulator takes per 16 spectra at most 6 MMAs on a diagonal tile
@@ -58,7 +58,10 @@ def rel(a, b):
 # pairs, 768 in fives with a remainder, 31 stations in pairs; 64 stations fill a
 # tile, 65 to 130 need off-diagonal ones and ragged last blocks
 SHAPES = [(1, 1, 16, 128), (8, 5, 64, 129), (8, 3, 256, 130), (31, 7, 64, 143), (32, 5, 64, 384), (33, 1, 64, 400),
-          (64, 1, 16, 1537), (65, 1, 16, 385), (76, 2, 16, 200), (130, 1, 16, 1536)]
+          (64, 1, 16, 1537), (65, 1, 16, 385), (76, 2, 16, 200), (130, 1, 16, 1536),
+          # few channels: time segments share a tile (8 of 96, 2 of 208, 4 of 240 with the
+          # last one short, 2 of a block that ends inside the first of the second's stages)
+          (8, 1, 64, 768), (24, 1, 16, 385), (13, 2, 16, 900), (3, 1, 16, 131)]
 
 
 @pytest.mark.parametrize("N,SB,C,S", SHAPES)
