@@ -73,13 +73,13 @@
 // visibility entry is owned by one lane of one CTA, which issues its chunks in
 // order, so the sum order is fixed and results are reproducible.
 //
-// Warp roles (persistent, one CTA per SM, 448 threads):
+// Warp roles (persistent, one CTA per SM, 512 threads):
 //   warp 0      TMA producer
 //   warp 1      TMEM allocator + MMA issuer (tcgen05.mma kind::tf32 and
 //               kind::f16 with BF16 operands, into the same accumulator)
 //   warps 2-9   epilogue: two warps per TMEM lane quadrant (warp % 4), each
 //               taking every other 32-column group of the upper triangle
-//   warps 10-13 converter
+//   warps 10-15 converter, two groups of three warps that take stages in turn
 // Two accumulators of 256 columns (double buffered) fill the 512 TMEM columns.
 // Every mbarrier wait is bounded; on expiry the role is recorded in the status
 // word, all roles leave, in-flight copies and MMAs are drained (bounded) and
@@ -99,7 +99,8 @@ namespace {
 
 using namespace tc;
 
-constexpr int kT3Threads = 448;
+constexpr int kT3Threads = 512;
+constexpr int kT3ConvGroups = 2, kT3ConvWarps = 3;    // converter: groups take stages in turn, a group's warps share one
 constexpr int kT3EpiWarps = 8;
 constexpr int kT3ConvWarp0 = 2 + kT3EpiWarps;
 constexpr int kT3K = 16;                              // spectra per stage (64-byte FP32 rows)
@@ -226,13 +227,13 @@ __device__ __forceinline__ uint2 neg_bf16x4(uint2 v) { return make_uint2(v.x ^ 0
 // hi J, -hi R, lo R, lo J, -lo R; for the row operand of an off-diagonal item
 // BF16 hi R, hi J, lo R, lo J.
 // W: the raw rows are first multiplied by the thread's four spectra's weights w
-// (the chunks a thread takes, t + 128 k, all hold the same four spectra).
+// (the chunks a thread takes, t + 96 k, all hold the same four spectra).
 template <bool W>
 __device__ __forceinline__ void convert_split(unsigned char *tf, unsigned tf_pitch, unsigned char *bf,
                                               unsigned bf_pitch, int rows, bool col, int t, float4 w)
 {
     const int nq = rows * (int)(kT3RowBytes / 16);
-    for (int q = t; q < nq; q += 128) {
+    for (int q = t; q < nq; q += 32 * kT3ConvWarps) {
         uint4 x = reinterpret_cast<const uint4 *>(tf)[q];
         uint4 y = reinterpret_cast<const uint4 *>(tf + tf_pitch)[q];
         if constexpr (W) {
@@ -293,7 +294,7 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_tf32_kernel(const __grid_
     if (threadIdx.x == 0) {
         for (int s = 0; s < P.stages; ++s) {
             mbar_init(full_bar(s), 1);
-            mbar_init(conv_bar(s), 4);              // one arrival per converter warp
+            mbar_init(conv_bar(s), kT3ConvWarps);   // one arrival per converter warp of the stage's group
             mbar_init(empty_bar(s), 1);
         }
         for (int b = 0; b < 2; ++b) {
@@ -367,6 +368,9 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_tf32_kernel(const __grid_
         // ================= MMA issuer =================
         if (lane == 0) {
             Ring ring;
+            // descriptors are built once; a plane, stage or K-step further on is an addition
+            // in 16-byte units (one thread issues every MMA)
+            const unsigned long long tdesc0 = sdesc64(tiles_u32), bdesc0 = sdesc32(tiles_u32);
             unsigned acc_it = 0;
             bool ok = true, issued = false;
             for (long long w = blockIdx.x; w < P.n_items && ok; w += gridDim.x) {
@@ -392,28 +396,26 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_tf32_kernel(const __grid_
                             break;
                         }
                         tc_fence_after();
-                        const unsigned st = tiles_u32 + (unsigned)s * P.stage_bytes;
-                        const unsigned bb = diag ? st : st + P.a_off;      // TF32 hi R, hi J, -hi R
-                        const unsigned bf = bb + 3 * pitch;                 // BF16 hi R, hi J, -hi R, lo R, lo J, -lo R
-                        // A planes: TF32 hi R, hi J; BF16 hi R, hi J, lo R, lo J
-                        const unsigned a_hr = diag ? bb : st;
-                        const unsigned a_hj = diag ? bb + pitch : st + kT3APlane;
-                        const unsigned a_bhr = diag ? bf : st + kT3ABf;
-                        const unsigned a_bhj = diag ? bf + bpitch : st + kT3ABf + kT3ABfPlane;
-                        const unsigned a_blr = diag ? bf + 3 * bpitch : st + kT3ABf + 2 * kT3ABfPlane;
-                        const unsigned a_blj = diag ? bf + 4 * bpitch : st + kT3ABf + 3 * kT3ABfPlane;
+                        const unsigned so = (unsigned)s * (P.stage_bytes >> 4), bo = diag ? 0u : P.a_off >> 4;
+                        const unsigned tp = pitch >> 4, bp = bpitch >> 4;
+                        // columns: TF32 hi R, hi J, -hi R, then BF16 hi R, hi J, -hi R, lo R, lo J, -lo R
+                        const unsigned long long bb = tdesc0 + so + bo, bf = bdesc0 + so + bo + 3 * tp;
+                        // rows: TF32 hi R, hi J; BF16 hi R, hi J, lo R, lo J
+                        constexpr unsigned AT = kT3APlane / 16, AB = kT3ABfPlane / 16, A0 = kT3ABf / 16;
+                        const unsigned long long a_hr = tdesc0 + so, a_hj = a_hr + (diag ? tp : AT);
+                        const unsigned long long ab0 = bdesc0 + so + (diag ? 3 * tp : A0);
+                        const unsigned long long a_bhj = ab0 + (diag ? bp : AB), a_blr = ab0 + (diag ? 3 * bp : 2 * AB);
+                        const unsigned long long a_blj = ab0 + (diag ? 4 * bp : 3 * AB);
 #pragma unroll
                         for (int kk = 0; kk < kT3K / 8; ++kk) {    // 8 FP32 = 32 bytes per TF32 K-step
-                            const unsigned acc = (kc | kk) ? 1u : 0u;
-                            const unsigned o = (unsigned)kk * 32u;
-                            mma_tf32(d, sdesc64(a_hr + o), sdesc64(bb + o), idesc, acc);           // [hi R; hi J]
-                            mma_tf32(d, sdesc64(a_hj + o), sdesc64(bb + pitch + o), idesc, 1u);    // [hi J; -hi R]
+                            mma_tf32(d, a_hr + 2u * kk, bb + 2u * kk, idesc, (kc | kk) ? 1u : 0u);   // [hi R; hi J]
+                            mma_tf32(d, a_hj + 2u * kk, bb + tp + 2u * kk, idesc, 1u);               // [hi J; -hi R]
                         }
                         // cross terms, K = 16 spectra in one BF16 MMA each
-                        mma_f16(d, sdesc32(a_bhr), sdesc32(bf + 3 * bpitch), idesc_bf, 1u);    // [lo R; lo J]
-                        mma_f16(d, sdesc32(a_bhj), sdesc32(bf + 4 * bpitch), idesc_bf, 1u);    // [lo J; -lo R]
-                        mma_f16(d, sdesc32(a_blr), sdesc32(bf), idesc_bf, 1u);                 // [hi R; hi J]
-                        mma_f16(d, sdesc32(a_blj), sdesc32(bf + bpitch), idesc_bf, 1u);        // [hi J; -hi R]
+                        mma_f16(d, ab0, bf + 3 * bp, idesc_bf, 1u);      // [lo R; lo J]
+                        mma_f16(d, a_bhj, bf + 4 * bp, idesc_bf, 1u);    // [lo J; -lo R]
+                        mma_f16(d, a_blr, bf, idesc_bf, 1u);             // [hi R; hi J]
+                        mma_f16(d, a_blj, bf + bp, idesc_bf, 1u);        // [hi J; -hi R]
                         issued = true;
                         mma_commit(empty_bar(s));
                     }
@@ -428,8 +430,10 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_tf32_kernel(const __grid_
         }
         __syncwarp();
     } else if (warp >= kT3ConvWarp0) {
-        // ================= converter (warps 10..13) =================
-        const int ct = threadIdx.x - kT3ConvWarp0 * 32; // 0..127
+        // ================= converter (warps 10..15) =================
+        const int grp = (warp - kT3ConvWarp0) / kT3ConvWarps;
+        const int ct = threadIdx.x - (kT3ConvWarp0 + grp * kT3ConvWarps) * 32;
+        int turn = 0;                                   // group of the next stage
         Ring ring;
         bool ok = true;
         for (long long w = blockIdx.x; w < P.n_items && ok; w += gridDim.x) {
@@ -437,9 +441,17 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_tf32_kernel(const __grid_
             const int n = itm.z;
             const bool diag = itm.w != 0;
             const unsigned pitch = (unsigned)n * kT3RowBytes;
-            for (int kc = 0; kc < P.nk; ++kc, ring.step(P.stages)) {
+            for (int kc = 0; kc < P.nk; ++kc) {
                 const int s = ring.i;
-                const bool got = t3wait(full_bar(s), ring.ph, abort_flag, P, 4);
+                const unsigned ph = ring.ph;
+                ring.step(P.stages);
+                const bool mine_now = turn == grp;
+                turn = turn + 1 == kT3ConvGroups ? 0 : turn + 1;
+                if (!mine_now) continue;
+                // the stage's last use first: the other group may have taken it, and the
+                // parity of the next wait would be ambiguous
+                const bool got = t3wait(empty_bar(s), ph ^ 1u, abort_flag, P, 4) &&
+                                 t3wait(full_bar(s), ph, abort_flag, P, 4);
                 if (!__all_sync(0xffffffffu, got)) {
                     ok = false;
                     break;
