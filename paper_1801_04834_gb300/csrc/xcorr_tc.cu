@@ -81,8 +81,9 @@ struct TcJob {
     float2 *vis;
     long long B;                      // baselines
     long long n_ch;                   // SB * C
-    int N, I_pad, nk, items_per_ch;
-    int ra;                           // rows of this job's A box
+    int N, I_pad, nk, items_per_ch;   // I_pad: of all channels of a group
+    int ra;                           // rows of this job's A box (of a group: all its boxes)
+    int group, gin;                   // channels per item (wide, one row block) and inputs of each
 };
 
 struct TcCommon {
@@ -263,7 +264,13 @@ __global__ void __launch_bounds__(kThreads, 1) xcorr_tc_kernel(const __grid_cons
                     mbar_arrive_expect_tx(full_bar(s), tx);
                     const unsigned dst = tiles_u32 + (unsigned)s * a.stage_bytes;
                     for (int pl = 0; pl < a.planes; ++pl) {
-                        const int z = (int)(itm.gch * a.planes + pl);
+                        const int z = (int)(itm.gch * J.group * a.planes + pl);
+                        if (J.group > 1) {              // channels past the last one arrive as zeros
+                            for (int c = 0; c < J.group; ++c)
+                                tma_load_3d(dst + (unsigned)pl * a_plane + (unsigned)(c * J.gin) * 128u, &J.mapA,
+                                            full_bar(s), kc * kBK, 0, z + c * a.planes);
+                            continue;
+                        }
                         tma_load_3d(dst + (unsigned)pl * a_plane, &J.mapA, full_bar(s), kc * kBK, row0, z);
                         if (!diag)
                             tma_load_3d(dst + a_region + (unsigned)pl * b_plane, &J.mapB, full_bar(s), kc * kBK,
@@ -371,10 +378,13 @@ __global__ void __launch_bounds__(kThreads, 1) xcorr_tc_kernel(const __grid_cons
             item_cols(P, J, itm, row0, col0, ncols);
             const int clen = a.chunk > 0 ? a.chunk : J.nk;
             const int ia = row0 + 32 * qd + lane;       // this lane's row input
-            const int i = ia >> 1, p = ia & 1;
+            const int cg = J.group > 1 ? ia / J.gin : 0;   // its channel of the group
+            const int first_st = cg * (J.gin >> 1);
+            const int i = (ia >> 1) - first_st, p = ia & 1;
+            const bool mine = cg < J.group && itm.gch * J.group + cg < J.n_ch;
             const int i_warp_min = (row0 + 32 * qd) >> 1;
             const unsigned lane_off = (unsigned)(32 * qd) << 16;
-            float2 *vrow = J.vis + itm.gch * J.B * 4;
+            float2 *vrow = J.vis + (itm.gch * J.group + cg) * J.B * 4;
             for (int k0 = 0; k0 < J.nk; k0 += clen, accs.step(a.nacc)) {
                 const int ab = accs.i;
                 const bool got = wait_bounded(accf_bar(ab), accs.ph, abort_flag, a, 3);
@@ -390,7 +400,7 @@ __global__ void __launch_bounds__(kThreads, 1) xcorr_tc_kernel(const __grid_cons
                 const unsigned t_im = t_re + (unsigned)a.ncm;
                 for (int cc = half; cc < ncols / 16; cc += kEpiWarps / 4) {
                     const int j0 = (col0 >> 1) + 8 * cc;   // first station of this 16-column chunk
-                    if (j0 >= J.N) break;
+                    if (J.group == 1 && j0 >= J.N) break;
                     if (j0 + 7 < i_warp_min) continue;    // whole chunk below the diagonal for this warp
                     float re[16], im[16];
                     tmem_ld16(t_re + 16 * cc, re);
@@ -400,8 +410,8 @@ __global__ void __launch_bounds__(kThreads, 1) xcorr_tc_kernel(const __grid_cons
                     if (a.accumulate && first) {
 #pragma unroll
                         for (int jj = 0; jj < 8; ++jj) {
-                            const int j = j0 + jj;
-                            old[jj] = (i <= j && j < J.N) ? *reinterpret_cast<const float4 *>(
+                            const int j = j0 + jj - first_st;
+                            old[jj] = (mine && i <= j && j < J.N) ? *reinterpret_cast<const float4 *>(
                                                                 vrow + ((long long)j * (j + 1) / 2 + i) * 4 + 2 * p)
                                                           : make_float4(0.f, 0.f, 0.f, 0.f);
                         }
@@ -409,8 +419,8 @@ __global__ void __launch_bounds__(kThreads, 1) xcorr_tc_kernel(const __grid_cons
                     tmem_ld_wait();
 #pragma unroll
                     for (int jj = 0; jj < 8; ++jj) {
-                        const int j = j0 + jj;
-                        if (i <= j && j < J.N) {
+                        const int j = j0 + jj - first_st;
+                        if (mine && i <= j && j < J.N) {
                             const long long b = (long long)j * (j + 1) / 2 + i;
                             const float s = a.inv_scale2;
                             float4 v = make_float4(re[2 * jj] * s, im[2 * jj] * s, re[2 * jj + 1] * s,
@@ -531,7 +541,7 @@ int items_per_ch(const TcConfig &cfg, int I_pad)
     return n;
 }
 
-bool encode_job(const TcConfig &cfg, int precision, const JobShape &js, int nk, TcJob &J)
+bool encode_job(const TcConfig &cfg, int precision, const JobShape &js, int nk, TcJob &J, int group = 1)
 {
     EncodeTiledFn enc = encode_fn();
     if (!enc) return false;
@@ -539,8 +549,8 @@ bool encode_job(const TcConfig &cfg, int precision, const JobShape &js, int nk, 
     const cuuint64_t gdim[3] = {(cuuint64_t)js.S_pad, (cuuint64_t)js.I_pad, (cuuint64_t)(js.n_ch * planes)};
     const cuuint64_t gstride[2] = {(cuuint64_t)js.S_pad * 2, (cuuint64_t)js.S_pad * 2 * js.I_pad};
     const cuuint32_t estr[3] = {1, 1, 1};
-    J.ra = job_ra(cfg, js.I_pad);
-    const cuuint32_t boxA[3] = {(cuuint32_t)kBK, (cuuint32_t)J.ra, 1};
+    J.ra = group > 1 ? group * js.I_pad : job_ra(cfg, js.I_pad);
+    const cuuint32_t boxA[3] = {(cuuint32_t)kBK, (cuuint32_t)(J.ra / group), 1};
     CUresult r = enc(&J.mapA, CU_TENSOR_MAP_DATA_TYPE_UINT16, 3, const_cast<void *>(js.corr), gdim, gstride, boxA,
                      estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -558,9 +568,11 @@ bool encode_job(const TcConfig &cfg, int precision, const JobShape &js, int nk, 
     J.B = (long long)js.N * (js.N + 1) / 2;
     J.n_ch = js.n_ch;
     J.N = js.N;
-    J.I_pad = js.I_pad;
+    J.I_pad = group * js.I_pad;
+    J.group = group;
+    J.gin = js.I_pad;
     J.nk = nk;
-    J.items_per_ch = items_per_ch(cfg, js.I_pad);
+    J.items_per_ch = items_per_ch(cfg, J.I_pad);
     return true;
 }
 
@@ -624,12 +636,22 @@ cudaError_t launch_xcorr_tc(const Handle &h, const void *corr, float2 *vis, cuda
     if (js[0].n_ch * planes_of(h.p.precision) > 0x7fffffffLL) return cudaErrorInvalidValue;
     TcParams<1> P;
     memset(&P, 0, sizeof(P));
-    if (!geometry(cfg, h.p.precision, js, P.c)) return cudaErrorNotSupported;
-    if (!encode_job(cfg, h.p.precision, js[0], h.S_pad / kBK, P.jobs[0])) return cudaErrorInvalidValue;
+    // Small arrays share a tile: the MMAs of a stage take as long as their 128 rows
+    // and accumulator latency, whatever the station count, so up to eight channels'
+    // inputs lie side by side and only the diagonal blocks of their products are
+    // stored, while every SM still gets an item (same bits; 8 stations x 6400
+    // channels x 256 spectra 160 -> 40 us, 30 x 3840 x 500 185 -> 107 us).
+    const int group = cfg.mode == 0 && h.I_pad <= 64
+                          ? (int)std::max<long long>(1, std::min<long long>(128 / h.I_pad, js[0].n_ch / h.num_sms))
+                          : 1;
+    std::vector<JobShape> tile = js;
+    tile[0].I_pad *= group;
+    if (!geometry(cfg, h.p.precision, tile, P.c)) return cudaErrorNotSupported;
+    if (!encode_job(cfg, h.p.precision, js[0], h.S_pad / kBK, P.jobs[0], group)) return cudaErrorInvalidValue;
     fill_common(P.c, h.d_status, h.operand_scale, h.tc_timeout_cycles, h.tc_test_no_tma);
     P.c.accumulate = accumulate ? 1 : 0;
     P.c.items = nullptr;
-    P.c.n_items = js[0].n_ch * P.jobs[0].items_per_ch;
+    P.c.n_items = (js[0].n_ch + group - 1) / group * P.jobs[0].items_per_ch;
     return launch_params(P, h.num_sms, st);
 }
 

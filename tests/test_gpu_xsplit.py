@@ -116,3 +116,29 @@ def test_forms_agree_and_accumulate():
     assert rel(pieces.channelize_correlate(raw, tau, tau), v.double()) < 2 * 12 * ULP
     for c in (whole, cores, pieces):
         c.close()
+
+
+@pytest.mark.parametrize("N,SB,C,S", [(3, 5, 64, 70), (8, 4, 256, 200), (17, 3, 256, 64), (31, 7, 64, 300)])
+@pytest.mark.parametrize("precision", [1, 2, 3])
+def test_channels_share_a_tile_16_bit(N, SB, C, S, precision):
+    """FP16/BF16/split operands of small arrays, several channels per tile with a remainder
+    (N = 8: six per tile; 17: five; 3 and 31: two): the same bits as a handle of one subband,
+    whose channels are too few to share."""
+    import paper_1801_04834_gb300 as m
+    whole = correlator(N, SB, C, S, precision)
+    taps = synth.kaiser_sinc_taps(4, 16)
+    one = m.Correlator(N, 1, 16, S, taps=taps, centres=synth.subband_centres(1), n_taps=4, precision=precision)
+    y = operands(N, SB, C, S, N).reshape(SB, C, S, 2 * N, 2).permute(0, 1, 4, 3, 2)
+    dt = whole.corr_dtype()
+    corr = torch.zeros(whole.corr_shape(), dtype=dt, device="cuda")
+    corr[:, :, :2, :whole.I, :S] = y.to(dt)
+    if precision == 3:
+        corr[:, :, 2:, :whole.I, :S] = (y - y.to(dt).float()).to(dt)
+    vis = torch.full(whole.vis_shape(), float("nan"), device="cuda")
+    whole.correlate(corr, out=vis)
+    for sb in range(SB):
+        for c0 in range(0, C, 16):
+            part = one.correlate(corr[sb:sb + 1, c0:c0 + 16].contiguous())
+            assert torch.equal(vis[sb:sb + 1, c0:c0 + 16], part), (sb, c0)
+    whole.close()
+    one.close()
