@@ -12,7 +12,8 @@ per-station bandpass ripple, 16-tap PPF to 64 channels, 3072 spectra per block
 (1.00663 s of sky), FP32-accurate path: the X-stage runs on the tcgen05 tensor
 cores with each FP32 operand split into hi + lo, hi hi' as TF32 MMAs and the
 cross terms hi lo' + lo hi' as BF16 MMAs (FX_TF32_SPLIT).
-The CUDA-core FFMA FP32 X-stage and the FP16 / BF16 / split-FP16 tensor-core
+The default precision (FX_F32, the same split on the spectrum-blocked layout),
+the CUDA-core FFMA FP32 X-stage and the FP16 / BF16 / split-FP16 tensor-core
 X-stages are timed on the same block, and the 8-bit precision workload (64
 stations, 488 subbands, 256 channels, 768 spectra) is timed at its own shape;
 every result's error is stated against the FP64 oracle on sampled subbands of
@@ -57,9 +58,9 @@ WORKLOADS = {
                               "hi lo' + lo hi' in BF16): "
                               "64 stations x 2 pols, 244 subbands, 16-tap PPF to 64 channels, "
                               "3072 spectra (1.00663 s) per block"),
-    "lofar16_ffma": dict(N=64, SB=244, C=64, S=3072, T=16, fmt=0, precision=0, sigma=100.0,
+    "lofar16_f32": dict(N=64, SB=244, C=64, S=3072, T=16, fmt=0, precision=0, sigma=100.0,
                          ntones=3, ripple=True, seed_index=1,
-                         desc="LOFAR 16-bit, FP32 path with the CUDA-core FFMA X-stage: 64 stations x 2 pols, "
+                         desc="LOFAR 16-bit, default FP32 precision (FX_F32): 64 stations x 2 pols, "
                               "244 subbands, 16-tap PPF to 64 channels, 3072 spectra (1.00663 s) per block"),
     "lofar8_fp16": dict(N=64, SB=488, C=256, S=768, T=16, fmt=1, precision=1, sigma=20.0,
                         ntones=1, ripple=False, seed_index=2,
@@ -68,9 +69,9 @@ WORKLOADS = {
     "lofar16_fp32_small": dict(N=64, SB=8, C=64, S=3072, T=16, fmt=0, precision=4, sigma=100.0,
                                ntones=3, ripple=True, seed_index=1,
                                desc="LOFAR 16-bit FP32-accurate path on 8 subbands (profiling size, ~4 GB)"),
-    "lofar16_ffma_small": dict(N=64, SB=8, C=64, S=3072, T=16, fmt=0, precision=0, sigma=100.0,
+    "lofar16_f32_small": dict(N=64, SB=8, C=64, S=3072, T=16, fmt=0, precision=0, sigma=100.0,
                                ntones=3, ripple=True, seed_index=1,
-                               desc="LOFAR 16-bit FFMA FP32 path on 8 subbands (profiling size, ~4 GB)"),
+                               desc="LOFAR 16-bit default FP32 path on 8 subbands (profiling size, ~4 GB)"),
     "lofar8_fp16_small": dict(N=64, SB=16, C=256, S=768, T=16, fmt=1, precision=1, sigma=20.0,
                               ntones=1, ripple=False, seed_index=2,
                               desc="LOFAR 8-bit FP16 X-stage on 16 subbands (profiling size, ~2.5 GB)"),
@@ -79,7 +80,7 @@ WORKLOADS = {
                       desc="8 stations x 2 pols, 1 subband, 64 channels, 768 spectra"),
 }
 
-PRECISION_NAMES = {0: "fp32_ffma", 1: "fp16", 2: "bf16", 3: "split_fp16", 4: "tf32_split"}
+PRECISION_NAMES = {0: "fp32", 1: "fp16", 2: "bf16", 3: "split_fp16", 4: "tf32_split"}
 DTYPE_NAMES = {0: "f32", 1: "f16", 2: "bf16", 3: "f16 hi+lo", 4: "f32 as hi+lo: tf32 hi hi', bf16 cross terms"}
 FP32_LANES_PER_SM = 128
 SM_MAX_MHZ = 2070.0
@@ -109,19 +110,37 @@ def tf32_split_tiles(c):
 
 
 def executed_xflops_split(c, w):
-    """(TF32, BF16) tensor-core flops the TF32-split X-stage issues: per 16
-    spectra and item, 4 TF32 MMAs of 128 x 2n x 8 (hi hi') and 4 BF16 MMAs of
-    128 x 2n x 16 (hi lo' + lo hi'), 2 flop per multiply-add."""
+    """(TF32, BF16) tensor-core flops of the split with every product formed (the
+    moving-delay adjoint's correlations): per 16 spectra and item, 4 TF32 MMAs
+    of 128 x 2n x 8 (hi hi') and 4 BF16 MMAs of 128 x 2n x 16 (hi lo' + lo hi'),
+    2 flop per multiply-add."""
     per_sp = tf32_split_tiles(c) * c.S_pad * w["C"] * w["SB"]
     return 4.0 * per_sp, 8.0 * per_sp
+
+
+def executed_xflops_half(c, w):
+    """(TF32, BF16) tensor-core flops the FP32-accurate X-stage issues: as
+    executed_xflops_split off the diagonal; a diagonal item of n inputs forms
+    3 of the 4 real products of hi hi' and one of the two cross terms."""
+    t = b = 0
+    for row0 in range(0, c.I_pad, 128):
+        n = min(128, c.I_pad - row0)
+        t += 128 * 3 * n
+        b += 128 * 4 * n
+        for c0 in range(row0 + 128, c.I_pad, 64):
+            n = min(64, c.I_pad - c0)
+            t += 128 * 4 * n
+            b += 128 * 8 * n
+    sp = (w["S"] + 15) // 16 * 16 * w["C"] * w["SB"]
+    return 2.0 * t * sp, 2.0 * b * sp
 
 
 def executed_xflops(c, w, precision):
     """Tensor-core flops the X-stage issues: 2 x 128 x N x K per MMA. FP16/BF16:
     4 real products of the I_pad x I_pad tile per spectrum (both triangles);
-    split FP16: 12; TF32 split: the TF32 and BF16 flops together."""
-    if precision == 4:
-        return sum(executed_xflops_split(c, w))
+    split FP16: 12; FP32-accurate split: the TF32 and BF16 flops together."""
+    if precision in (0, 4):
+        return sum(executed_xflops_half(c, w))
     ip, sp = c.I_pad, c.S_pad
     nch = w["C"] * w["SB"]
     mult = {1: 4, 2: 4, 3: 12}[precision]
@@ -517,13 +536,13 @@ def run_fx(args, w):
     xflops = useful_xflops(w)
     sz = c.sizes
     x_ach = xflops / (ms_x * 1e-3) / 1e12
-    if prec == 4:
-        ex = executed_xflops_split(c, w)
+    if prec in (0, 4):
+        ex = executed_xflops_half(c, w)
         tpk, bpk = peaks_run["tf32_tflops"], peaks_run["bf16_tflops"]
         sr = split_roofline(xflops, ex, ms_x, tpk, bpk)
-        roof = {"kernel": "xcorr_tf32_kernel", "bound": "tensor", "achieved": sr["achieved"], "peak": tpk,
+        roof = {"kernel": "xcorr_split_kernel", "bound": "tensor", "achieved": sr["achieved"], "peak": tpk,
                 "unit": "TFLOP/s", "frac": sr["frac"],
-                "traffic": recorded_traffic("xcorr_tf32_kernel", args.workload),
+                "traffic": recorded_traffic("xcorr_split_kernel", args.workload),
                 "peak_source": "dense TF32 tensor throughput measured in this run (torch TF32 matmul 8192^3, "
                                "burst); MEASURED_PEAKS.json holds no TF32 figure; BF16 peak of the same run "
                                f"({bpk:.0f} TFLOP/s) for the BF16 part",
@@ -533,15 +552,8 @@ def run_fx(args, w):
                                f"floor {sr['floor_ms']:.2f} ms / measured {ms_x:.2f} ms",
                 "useful_fp32_equiv_TFLOPs": x_ach, "useful_frac": x_ach / tpk,
                 "executed_TFLOPs": sr["executed_TFLOPs"], "executed_frac": sr["executed_frac"],
-                "executed_note": "whole 128-input tiles (both triangles) are issued: %.2fx the algorithmic work"
+                "executed_note": "half the products of whole 128-input tiles (both triangles) are issued: %.2fx the algorithmic work"
                                  % (sr["executed_floor_ms"] / sr["floor_ms"])}
-    elif prec == 0:
-        fpk = fp32_alu_peak_tflops(sm_count)
-        roof = {"kernel": "xcorr_f32_kernel", "bound": "alu", "achieved": x_ach, "peak": fpk,
-                "unit": "TFLOP/s", "frac": x_ach / fpk,
-                "traffic": recorded_traffic("xcorr_f32_kernel", args.workload),
-                "peak_source": f"derived: {sm_count} SMs (device property) x 128 FP32 lanes x 2 flop x 2070 MHz",
-                "algorithmic": f"{xflops:.4e} useful flop per launch (8 per complex MAC)"}
     else:
         x_bytes = sz.corr_bytes + sz.vis_bytes
         xb = x_bytes / (ms_x * 1e-3) / 1e9
@@ -577,13 +589,13 @@ def run_fx(args, w):
     # F-stage writing its own operand layout; errors against the same oracle ----
     variants = {}
     if not args.no_variants:
-        for vp in (0, 4, 1, 2, 3):
-            if vp == prec:
+        for vp, form in VARIANTS:
+            if vp == prec and form == "auto":
                 continue
-            name = PRECISION_NAMES[vp]
+            name = variant_name(vp, form)
             try:
                 variants[name] = precision_variant(args, w, vp, raw, taps, centres, delays, bandpass, stream,
-                                                   sbs, ref)
+                                                   sbs, ref, form)
             except Exception as ex:  # report, do not hide
                 variants[name] = {"error": str(ex)[:200]}
         head = {"step_ms": ms_step, "correlate_ms": ms_x}
@@ -694,7 +706,15 @@ def run_fx(args, w):
     return 0
 
 
-def precision_variant(args, w, vp, raw, taps, centres, delays, bandpass, stream, sbs, ref):
+# X-stage forms timed beside the headline: (precision, FP32 form); "2x4" is the CUDA-core X-stage
+VARIANTS = ((4, "auto"), (0, "auto"), (0, "2x4"), (1, "auto"), (2, "auto"), (3, "auto"))
+
+
+def variant_name(vp, form):
+    return PRECISION_NAMES[vp] + ("_ffma" if form != "auto" else "")
+
+
+def precision_variant(args, w, vp, raw, taps, centres, delays, bandpass, stream, sbs, ref, form="auto"):
     """One X-stage precision on a resident raw block: the fused F-stage in that
     precision's operand layout + the X-stage, timed as a step and alone, with
     the error of the result against the oracle visibilities `ref` of `sbs`."""
@@ -703,7 +723,7 @@ def precision_variant(args, w, vp, raw, taps, centres, delays, bandpass, stream,
     import paper_1801_04834_gb300 as fxg
     dev = raw.device
     cv = fxg.Correlator(w["N"], w["SB"], w["C"], w["S"], taps=taps, centres=centres, n_taps=w["T"],
-                        fmt=w["fmt"], precision=vp)
+                        fmt=w["fmt"], precision=vp, xf32_form=form)
     corr_v = torch.empty(cv.corr_shape(), dtype=cv.corr_dtype(), device=dev)
     vis_v = torch.empty(cv.vis_shape(), dtype=torch.float32, device=dev)
 
@@ -729,7 +749,7 @@ def precision_variant(args, w, vp, raw, taps, centres, delays, bandpass, stream,
     out = {"step_ms": step_ms, "step_rtf": sky_seconds(w) / (step_ms * 1e-3),
            "channelize_correct_ms": f_ms, "channelize_correct_hbm_frac": fc_bytes / (f_ms * 1e-3) / 1e9 / hbm,
            "correlate_ms": x_ms, "correlate_useful_TFLOPs": xflops / (x_ms * 1e-3) / 1e12}
-    if vp != 0:
+    if form == "auto":
         ex = executed_xflops(cv, w, vp)
         out["correlate_executed_TFLOPs"] = ex / (x_ms * 1e-3) / 1e12
     if vp in (1, 2, 3):
@@ -757,10 +777,10 @@ def measure_precision_form(args, dev):
     sbs = [1, w["SB"] - 2]
     ref = None if args.no_parity else oracle_reference(w, raw, taps, centres, tau, ripple, sbs)
     res = {"workload": w["desc"], "subbands_checked": sbs}
-    for vp in (4, 0, 1, 2, 3):
-        name = PRECISION_NAMES[vp]
+    for vp, form in VARIANTS:
+        name = variant_name(vp, form)
         try:
-            res[name] = precision_variant(args, w, vp, raw, taps, centres, delays, bandpass, stream, sbs, ref)
+            res[name] = precision_variant(args, w, vp, raw, taps, centres, delays, bandpass, stream, sbs, ref, form)
         except Exception as ex:
             res[name] = {"error": str(ex)[:200]}
         torch.cuda.empty_cache()

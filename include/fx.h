@@ -126,9 +126,10 @@ typedef struct {
  * samples, and allocates one assembled raw block as workspace. */
 #define FX_FLAG_STREAMING 0x1u
 
-/* Tuning hints for the FP32 X-stage (results agree up to FP32 rounding
- * order). Default: 4 x 4-station register tiles from 16 stations up (2 x 4
- * below). SMALL: 2 x 4 tiles. THREE_MULT: 2 x 4 tiles with the
+/* Forms of the FP32 X-stage (results agree up to FP32 rounding). Default: the
+ * tensor cores from 128 spectra on (fx_correlate), else the CUDA cores with
+ * 4 x 4-station register tiles from 16 stations up (2 x 4 below). SMALL: the
+ * CUDA cores with 2 x 4 tiles. THREE_MULT: the same with the
  * three-multiplication complex product (sum xr yr, sum xi yi,
  * sum (xr + xi)(yr - yi)): 3 FMAs per complex MAC instead of 4. */
 #define FX_FLAG_XF32_SMALL_TILES 0x2u
@@ -208,14 +209,17 @@ fx_status fx_channelize_correct(fx_handle *h, const void *d_raw, const double *d
 /* X-stage correlation (Sec. "Signal processing with GPU kernels": the last
  * kernel correlates all pairs of antenna fields and integrates ~1 s):
  *   vis[sb][k][b(i,j)][2p+q] = sum_{s<S} Y[i,p] conj(Y[j,q])  for i <= j.
- * d_corr: corr layout of the handle's precision; d_vis: vis layout. FP32
- * operands run on the CUDA cores; FP16/BF16/split operands on the tcgen05
- * tensor cores with FP32 accumulation (split: hi*hi' + hi*lo' + lo*hi',
- * accumulator chains restarted every 256 spectra and summed in IEEE FP32);
- * FX_TF32_SPLIT operands (FP32 planar) on the tcgen05 tensor cores as hi/lo
- * parts (hi*hi' in TF32, the cross terms in BF16) with FP32 accumulation,
- * accumulator chains restarted every 64 spectra and summed in IEEE FP32 (FP32
- * accuracy, any station count up to 512; results reproducible run to run). */
+ * d_corr: corr layout of the handle's precision; d_vis: vis layout.
+ * FP16/BF16/split operands run on the tcgen05 tensor cores with FP32
+ * accumulation (split: hi*hi' + hi*lo' + lo*hi', accumulator chains restarted
+ * every 256 spectra and summed in IEEE FP32). FX_TF32_SPLIT operands (FP32
+ * planar) run there as hi/lo parts (hi*hi' in TF32, the cross terms in BF16)
+ * with FP32 accumulation, accumulator chains of 64 spectra summed in IEEE FP32
+ * (FP32 accuracy, any station count up to 512; results reproducible run to
+ * run). FX_F32 operands take the same form from 128 spectra on (chains of 16 to
+ * 64 spectra, by the block's length: no less accurate than an FP32 FMA chain
+ * over it), and FP32 FMAs on the CUDA cores below that, above 512 stations, and
+ * where an FX_FLAG_XF32_* flag asks for a form of those. */
 fx_status fx_correlate(fx_handle *h, const void *d_corr, float *d_vis, fx_stream stream);
 
 /* End to end from host memory: raw samples in, visibilities out, for all
@@ -364,7 +368,7 @@ fx_status fx_correct_correlate_backward(fx_handle *h, const float *d_raw_vis, co
  * and dV_ab/dtau_begin = +-i 2 pi f_k g_a conj(g_b) (K_ab - M1_ab) (+ for the
  * first station of the entry, - for the second). The call recomputes Y from
  * the channelised block (d_chan, chan layout) into d_work_corr (corr layout
- * of the handle's precision, caller-owned, corr_bytes of fx_query_sizes,
+ * of the handle's precision, caller-owned, overwritten, corr_bytes of fx_query_sizes,
  * 128-byte aligned), forms K and M1 with the X-stage into d_work_vis
  * (2 x vis_bytes, caller-owned; K first) and writes d_grad_gains [N][P]
  * complex float, d_grad_delay_begin [N] and d_grad_delay_end [N] double

@@ -283,12 +283,7 @@ __global__ void adjoint_interp_partial_kernel(const float2 *__restrict__ K, cons
 int adjoint_blocks(const Handle &h)
 {
     const long long total = (long long)h.p.n_subbands * h.p.n_channels;
-    // one channel per CTA while there are few: the per-channel loop is a serial chain
-    // of loads, so what counts is how many CTAs share an SM (76 stations x 2048
-    // channels, moving delays: 217 us with 2048 CTAs, 421 with two per SM)
-    const long long sms = h.num_sms > 0 ? h.num_sms : 152;
-    const long long fit = (16LL << 20) / (4 * (long long)sizeof(double) * h.I);   // 16 MB of partials
-    const long long want = fit > 16 * sms ? 16 * sms : fit > 2 * sms ? fit : 2 * sms;
+    const long long want = 2LL * (h.num_sms > 0 ? h.num_sms : 152);
     return (int)(total < want ? total : want);
 }
 
@@ -340,19 +335,22 @@ cudaError_t launch_weight_spectra(const Handle &h, float2 *corr, cudaStream_t st
 }
 
 cudaError_t launch_adjoint_interp(const Handle &h, const float2 *K, const float2 *M1, const float2 *G,
-                                  const float2 *gains, float2 *grad_gains, double *grad_tb, double *grad_te,
-                                  cudaStream_t st)
+                                  const float2 *gains, double *partial, float2 *grad_gains, double *grad_tb,
+                                  double *grad_te, cudaStream_t st)
 {
     const int I = h.I;
     if (I > 1024) return cudaErrorNotSupported;
     const long long total = (long long)h.p.n_subbands * h.p.n_channels;
-    const int nblk = adjoint_blocks(h);
+    // one channel per CTA while there are few: the per-channel loop is a serial chain
+    // of loads, so what counts is how many CTAs share an SM (76 stations x 2048
+    // channels: 217 us with 2048 CTAs, 421 with two per SM)
+    const int nblk = (int)(total < 16LL * h.num_sms ? total : 16LL * h.num_sms);
     const int threads = (I + 31) / 32 * 32;
     adjoint_interp_partial_kernel<<<nblk, threads, sizeof(float2) * I, st>>>(
-        K, M1, G, gains, h.d_centres, h.d_adj_partial, h.p.n_stations, h.p.n_channels, total, h.p.sample_rate_hz);
+        K, M1, G, gains, h.d_centres, partial, h.p.n_stations, h.p.n_channels, total, h.p.sample_rate_hz);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    adjoint_reduce_kernel<4><<<h.p.n_stations, kRedThreads, 0, st>>>(h.d_adj_partial, nblk, h.p.n_stations,
+    adjoint_reduce_kernel<4><<<h.p.n_stations, kRedThreads, 0, st>>>(partial, nblk, h.p.n_stations,
                                                                      grad_gains, grad_tb, grad_te);
     return cudaGetLastError();
 }

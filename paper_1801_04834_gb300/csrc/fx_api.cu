@@ -570,9 +570,11 @@ extern "C" fx_status fx_correct_correlate_backward_interp(
     if (e == cudaSuccess) e = adjoint_xstage(*h, d_work_corr, K, false, s);           // K = sum Y Y^H
     if (e == cudaSuccess) e = adjoint_xstage(*h, d_work_corr, M1, true, s);           // M1 = sum (s/S) Y Y^H
     if (e == cudaSuccess)
+        // the corrected block is done with: its buffer takes the partial sums (4 doubles
+        // per channel and input at most; it holds 16 spectra or more of each)
         e = fxi::launch_adjoint_interp(*h, K, M1, reinterpret_cast<const float2 *>(d_grad_vis),
                                        reinterpret_cast<const float2 *>(d_gains),
-                                       reinterpret_cast<float2 *>(d_grad_gains), d_grad_delay_begin,
+                                       static_cast<double *>(d_work_corr), reinterpret_cast<float2 *>(d_grad_gains), d_grad_delay_begin,
                                        d_grad_delay_end, s);
     return after_launch(e, who);
 }

@@ -93,9 +93,10 @@ cudaError_t launch_apply_gains(const Handle &h, const float2 *R, const float2 *g
 cudaError_t launch_adjoint(const Handle &h, const float2 *R, const float2 *G, const float2 *gains,
                            const double *tau, float2 *grad_gains, double *grad_tau, cudaStream_t st);
 cudaError_t launch_weight_spectra(const Handle &h, float2 *corr, cudaStream_t st);   // FX_F32 layout, in place
+// partial: room for 4 doubles per (channel, input), at most 16 channels per SM
 cudaError_t launch_adjoint_interp(const Handle &h, const float2 *K, const float2 *M1, const float2 *G,
-                                  const float2 *gains, float2 *grad_gains, double *grad_tb, double *grad_te,
-                                  cudaStream_t st);
+                                  const float2 *gains, double *partial, float2 *grad_gains, double *grad_tb,
+                                  double *grad_te, cudaStream_t st);
 
 // beamform.cu
 size_t bf_weight_bytes(const Handle &h, int n_beams);

@@ -1,4 +1,9 @@
-// xcorr_f32.cu -- X-stage correlator in FP32 on the CUDA cores (FFMA).
+// xcorr_f32.cu -- X-stage correlator in FP32 on the CUDA cores (FFMA): FX_F32
+// below 128 spectra, above 512 stations, where a flag asks for one of these
+// forms, and the correlations of the FX_F32 moving-delay adjoint (whose FP64
+// gradients keep their rounding). Everything else of FX_F32 runs in
+// xcorr_split.cu, which is four to five times as fast at 64 stations and closer
+// to FP64 from 128 spectra on.
 //
 // Paper, Sec. "Signal processing with GPU kernels": the last kernel correlates
 // all pairs of antenna fields and integrates to ~1 s. Sec. "Hardware
