@@ -672,23 +672,32 @@ __global__ void __launch_bounds__(256) planar_pad_kernel(uint4 *__restrict__ cor
 // FFT threads in two groups of 128. A round's rows (16 spectra of one input) fit
 // twice in shared memory at this channel count only per input; the CTAs of a
 // station's two pols are neighbours in the grid and read the same raw rows (the
-// second read mostly from L2). FIR round b -> u[b & 1] -> FULL[b & 1]; FFT group
-// g takes the rounds b = g mod 2 (row buffer g) with its own named barrier, so
-// two rounds are in FFT at once.
+// second read mostly from L2). FIR round b -> u[b % NB] -> FULL[b % NB]; FFT group
+// g takes the rounds b = g mod 2 with its own named barrier, so two rounds are in
+// FFT at once.
 //
 // What bounds it: the FMA pipe with the register reads of its packed FMAs. The
 // FIR alone (16 warps, nothing else running) takes 2.0 ms of the 8-bit case below,
 // 0.64 of the pipe's rate in every instruction order tried, and the FFT's adds and
 // multiplies 1.4 ms at full rate, 3.4 ms together; more warps (20, 24) gain
 // nothing. So the design saves instructions and shared-memory traffic:
-//  * the phase factors come from the channel axis. f_k is linear in k, so for a
-//    spectrum s exp(i phi(k, s)) = e(k1, s) r(s)^m for k = k1 + 128 + 16 m: the
-//    FIR threads put one anchor e (16 x 16 per round, each the gain, flag and
-//    scale times one __sincosf) into a table, the phase-table kernel has left
-//    r(s) = exp(2 pi i (fs / 16) tau(s)) per station and spectrum, and an FFT
-//    thread steps from its anchor up and down eight channels each in registers.
-//    (One entry per channel and spectrum, rotated along time by the FIR threads,
-//    took a 70 KB table and a store and a load per output.)
+//  * FP32 and split FP16: the phase factors come from the channel axis. f_k is
+//    linear in k, so for a spectrum s exp(i phi(k, s)) = e(k1, s) r(s)^m for
+//    k = k1 + 128 + 16 m: the FIR threads put one anchor e (16 x 16 per round,
+//    each the gain, flag and scale times one __sincosf) into a table, the
+//    phase-table kernel has left r(s) = exp(2 pi i (fs / 16) tau(s)) per station
+//    and spectrum, and an FFT thread steps from its anchor up and down eight
+//    channels each in registers.
+//  * FP16 and BF16 (TIME): one factor per channel and spectrum, an anchor per
+//    channel and round rotated along time by the channel's FIR thread. The two
+//    ways differ by 3e-7, as little as either from the exact factor, but in a
+//    16-bit operand that flips a rounding now and then, and a beam voltage, which
+//    averages nothing, then moves by a unit of the operand (4e-5 normwise in
+//    BF16): what users of these precisions have stored would no longer come out
+//    again. It costs a 37 KB table per buffer, hence two row buffers, and 4.38 ms
+//    instead of 4.01 in the 8-bit case below. The chain of rotations stands beside
+//    the second half of the FIR, and the table is freed after the row buffer (in
+//    one piece before the FIR, and freed with it: 4.47 ms).
 //  * pass 1 (row = 16 lanes) writes its results transposed, P1[k1][n2][row] over
 //    u[g] after the group's barrier; in pass 2 a thread takes two adjacent
 //    spectra of one k1, so P1 rows come in 16-byte loads and planar values leave
@@ -696,10 +705,14 @@ __global__ void __launch_bounds__(256) planar_pad_kernel(uint4 *__restrict__ cor
 //  * strides: FIR rows 264 (two rows' halves fall on both halves of the banks in
 //    pass 1), P1 rows 18 (even, for the 16-byte loads; eight n2 x two rows of a
 //    store on distinct banks).
-// 64 stations, 61 subbands of int8, 768 spectra, FP16 out: 4.45 -> 4.16 ms (2.2
-// TB/s of raw rows and operands); two row buffers instead of four 4.34 ms; with
-// the FIR's eight outputs at a time 4.01 ms.
+// 64 stations, 61 subbands of int8, 768 spectra, before this form -> now: FP32
+// planes 4.44 -> 4.13 ms (3.7 TB/s of raw rows and operands), FP16 4.45 -> 4.38
+// ms. With
+// anchors, two row buffers instead of four took 4.34 for 4.16 ms, four FIR
+// outputs at a time instead of eight 4.16 for 4.01.
+template <int OUT>
 struct Ws256 {
+    static constexpr bool TIME = OUT <= 3;              // factors along time (16-bit operands)
     static constexpr int C = 256, R = 16;
     static constexpr int NF = C, NG = 128;              // FIR threads; FFT threads of a group
     static constexpr int ALL = NF + 2 * NG;
@@ -707,14 +720,15 @@ struct Ws256 {
     static constexpr int RS = kRound + 2;               // P1 row stride
     static constexpr int USZ = R * R * RS > kRound * ROW ? R * R * RS : kRound * ROW;   // one buffer: 16 rows, then P1
     static constexpr int TW = R + 2;                    // twiddle row: [n2][k1], even
-    static constexpr int ESZ = R * kRound;              // anchors [k1][spectrum] of a round
-    static constexpr int NB = 4;                        // row buffers
+    static constexpr int EJ = kRound + 2;               // row of a factor table (even, conflict-free in 16 bytes)
+    static constexpr int ESZ = TIME ? C * EJ : R * kRound;   // factors [channel][spectrum], or anchors [k1][spectrum]
+    static constexpr int NB = TIME ? 2 : 4;             // row buffers
 };
 
-template <typename TIn>
+template <typename TIn, int OUT>
 constexpr size_t ws256_smem_bytes()
 {
-    using W = Ws256;
+    using W = Ws256<OUT>;
     return 2ull * kRound * W::C * kPols * sizeof(TIn) +
            ((size_t)W::NB * (W::USZ + W::ESZ) + (size_t)W::R * W::TW) * sizeof(float2) + W::C * sizeof(float2) + 16;   // + 2 mbarriers
 }
@@ -722,7 +736,7 @@ constexpr size_t ws256_smem_bytes()
 __device__ __forceinline__ float2 conj2(float2 a) { return make_float2(a.x, -a.y); }
 
 template <int T, typename TIn, int OUT>
-__global__ void __launch_bounds__(Ws256::ALL, 1)
+__global__ void __launch_bounds__(Ws256<OUT>::ALL, 1)
 ppf_correct_ws256_kernel(const TIn *__restrict__ raw, void *__restrict__ corr, const float *__restrict__ taps,
                          const float2 *__restrict__ twiddle, const float2 *__restrict__ phase,
                          const float2 *__restrict__ ratio, const float *__restrict__ bandpass,
@@ -730,20 +744,22 @@ ppf_correct_ws256_kernel(const TIn *__restrict__ raw, void *__restrict__ corr, c
                          int rounds_per_cta, const float *__restrict__ flags, int s_base, int s_end,
                          int *__restrict__ status, long long budget, int no_loads)
 {
-    using W = Ws256;
+    using W = Ws256<OUT>;
     constexpr int C = W::C, R = W::R, NF = W::NF, ROW = W::ROW, USZ = W::USZ, RS = W::RS, TW = W::TW, ESZ = W::ESZ;
+    constexpr bool TIME = W::TIME;
+    constexpr int EJ = W::EJ;
     constexpr int ROW_BYTES = C * kPols * (int)sizeof(TIn);     // one raw time row of the station (both pols)
     constexpr int BUF_BYTES = kRound * ROW_BYTES;
     constexpr int NG = W::NG;
     constexpr int HAND = NF + NG;               // FULL / EMPTY: the FIR threads and one FFT group
     static_assert(OUT >= 2 && OUT <= 5, "planar outputs");
     static_assert(ROW_BYTES % 16 == 0, "rows must be whole 16-byte chunks");
-    static_assert(ws256_smem_bytes<TIn>() <= 227 * 1024, "one CTA per SM");
+    static_assert(ws256_smem_bytes<TIn, OUT>() <= 227 * 1024, "one CTA per SM");
 
     extern __shared__ __align__(16) unsigned char smem[];
     unsigned char *inbuf = smem;
     float2 *u = reinterpret_cast<float2 *>(inbuf + 2 * BUF_BYTES);   // [NB][USZ]
-    float2 *et = u + W::NB * USZ;                                     // [NB][k1][spectrum] anchors
+    float2 *et = u + W::NB * USZ;                                     // [NB][ESZ] factors or anchors
     float2 *tw = et + W::NB * ESZ;                                        // [n2][TW] W_C^(n2 k1)
     float2 *bpt = tw + R * TW;                                        // [k1][k2] bandpass of output k2, twice
     const unsigned rbar = tc::smem_u32(bpt + C);                      // raw-row mbarriers [2]
@@ -784,9 +800,13 @@ ppf_correct_ws256_kernel(const TIn *__restrict__ raw, void *__restrict__ corr, c
         const int c = tid;
         // anchor role: channel k1 + 128 (k1 = c / 16) of spectrum c % 16 of a round
         const int aj = c % kRound;
-        const float2 pst = phase[((long long)sb * N + n) * C + C / 2 + c / kRound];   // (phi0, step)
+        // (with factors along time: channel c, from the round's first spectrum on)
+        const float2 pst = phase[((long long)sb * N + n) * C + (TIME ? c : C / 2 + c / kRound)];   // (phi0, step)
         const float2 gg = gains ? gains[n * kPols + p] : make_float2(1.f, 0.f);
-        const float2 gsc = make_float2(gg.x * scale, gg.y * scale);
+        const float bpc = TIME && bandpass ? bandpass[(long long)n * C + c] : 1.f;
+        const float2 gsc = make_float2(bpc * gg.x * scale, bpc * gg.y * scale);
+        float2 rot = make_float2(1.f, 0.f);
+        if constexpr (TIME) sincosf(pst.y, &rot.y, &rot.x);          // exp(i step)
         float2 h[T];
 #pragma unroll
         for (int k = 0; k < T; ++k) h[k] = make_float2(taps[k * C + c], taps[k * C + c]);
@@ -811,19 +831,19 @@ ppf_correct_ws256_kernel(const TIn *__restrict__ raw, void *__restrict__ corr, c
             // split of 2 pi), __sincosf, times gain, scale and flag
             float2 e;
             {
-                const float phi = fmaf((float)(sr + aj), pst.y, pst.x);
+                const float phi = fmaf((float)(TIME ? sr : sr + aj), pst.y, pst.x);
                 const float kq = rintf(phi * 0.15915494309189535f);
                 float r = fmaf(-kq, 6.28125f, phi);
                 r = fmaf(-kq, 1.9353071795864769e-3f, r);
                 __sincosf(r, &e.y, &e.x);
             }
             e = cmul(gsc, e);
-            if (flags) {
+            if (!TIME && flags) {
                 const float fw = flags[(long long)n * S + min(sr + aj, S - 1)];
                 e = make_float2(e.x * fw, e.y * fw);
             }
             if (b >= W::NB) named_bar_sync(kBar256Empty + ub, HAND);
-            et[ub * ESZ + c] = e;
+            if constexpr (!TIME) et[ub * ESZ + c] = e;
             const TIn *in = reinterpret_cast<const TIn *>(inbuf + q * BUF_BYTES);
             float2 *uq = u + ub * USZ;
             // eight outputs at a time, each sample's products one after the other: 4.01 ms
@@ -834,6 +854,20 @@ ppf_correct_ws256_kernel(const TIn *__restrict__ raw, void *__restrict__ corr, c
             constexpr int QN = 8;
 #pragma unroll
             for (int j0 = 0; j0 < kRound; j0 += QN) {
+                if constexpr (TIME) {
+                    // the factors along time beside the second half's FMAs; their table is
+                    // free later than the row buffer
+                    if (j0 == QN) {
+                        if (b >= W::NB) named_bar_sync(kBar256EmptyF + ub, HAND);
+                        float4 *eq = reinterpret_cast<float4 *>(et + ub * ESZ + c * EJ);
+#pragma unroll
+                        for (int j = 0; j < kRound; j += 2) {
+                            const float2 e1 = cmul(e, rot);
+                            eq[j / 2] = make_float4(e.x, e.y, e1.x, e1.y);
+                            e = cmul(e1, rot);
+                        }
+                    }
+                }
                 float2 t[QN], acc[QN];
 #pragma unroll
                 for (int qq = 0; qq < QN; ++qq) {
@@ -852,6 +886,13 @@ ppf_correct_ws256_kernel(const TIn *__restrict__ raw, void *__restrict__ corr, c
                 for (int qq = 0; qq < QN; ++qq) {
                     uq[(j0 + qq) * ROW + c] = acc[qq];
                     win[(T - 1 + j0 + qq) % T] = t[qq];
+                }
+            }
+            if (TIME && flags) {
+                float2 *eq = et + ub * ESZ + c * EJ;
+                for (int j = 0; j < kRound; ++j) {
+                    const float fw = flags[(long long)n * S + min(sr + j, S - 1)];
+                    eq[j] = make_float2(eq[j].x * fw, eq[j].y * fw);
                 }
             }
             named_bar_arrive(kBar256Full + ub, HAND);
@@ -875,7 +916,8 @@ ppf_correct_ws256_kernel(const TIn *__restrict__ raw, void *__restrict__ corr, c
             const int q = b % W::NB;
             const int sr = s0 + b * kRound;
             float2 *uq = u + q * USZ;
-            const float4 rr = *reinterpret_cast<const float4 *>(ratio + (long long)n * S16 + sr + jp);
+            float4 rr = make_float4(1.f, 0.f, 1.f, 0.f);
+            if constexpr (!TIME) rr = *reinterpret_cast<const float4 *>(ratio + (long long)n * S16 + sr + jp);
             named_bar_sync(kBar256Full + q, HAND);
             float2 v[2][R];
 #pragma unroll
@@ -905,30 +947,44 @@ ppf_correct_ws256_kernel(const TIn *__restrict__ raw, void *__restrict__ corr, c
                 v[0][m] = make_float2(w.x, w.y);
                 v[1][m] = make_float2(w.z, w.w);
             }
-            const float4 ee = *reinterpret_cast<const float4 *>(et + q * ESZ + k1 * kRound + jp);
-            if (b + W::NB < nrounds) named_bar_arrive(kBar256Empty + q, HAND);
+            if constexpr (TIME) {
+                if (b + W::NB < nrounds) named_bar_arrive(kBar256Empty + q, HAND);
 #pragma unroll
-            for (int it = 0; it < 2; ++it) fft_reg<R>(v[it]);
-            // output k2 is channel k1 + 128 + 16 k2 for k2 < 8 and k1 + 128 + 16 (k2 - 16) above
-            float2 r[2] = {make_float2(rr.x, rr.y), make_float2(rr.z, rr.w)};
-            float2 up[2] = {make_float2(ee.x, ee.y), make_float2(ee.z, ee.w)}, dn[2];
+                for (int it = 0; it < 2; ++it) fft_reg<R>(v[it]);
 #pragma unroll
-            for (int it = 0; it < 2; ++it) dn[it] = cmul(up[it], conj2(r[it]));
+                for (int k2 = 0; k2 < R; ++k2) {
+                    const int kout = k1 + R * ((k2 + R / 2) % R);
+                    const float4 f = *reinterpret_cast<const float4 *>(et + q * ESZ + kout * EJ + jp);
+                    v[0][k2] = cmul(v[0][k2], make_float2(f.x, f.y));
+                    v[1][k2] = cmul(v[1][k2], make_float2(f.z, f.w));
+                }
+                if (b + W::NB < nrounds) named_bar_arrive(kBar256EmptyF + q, HAND);
+            } else {
+                const float4 ee = *reinterpret_cast<const float4 *>(et + q * ESZ + k1 * kRound + jp);
+                if (b + W::NB < nrounds) named_bar_arrive(kBar256Empty + q, HAND);
 #pragma unroll
-            for (int k2 = 0; k2 < R / 2; k2 += 2) {
-                const float4 bu = *reinterpret_cast<const float4 *>(bpt + k1 * R + k2);
-                const float4 bd = *reinterpret_cast<const float4 *>(bpt + k1 * R + R - 2 - k2);
-                const float2 fu[2] = {make_float2(bu.x, bu.y), make_float2(bu.z, bu.w)};
-                const float2 fd[2] = {make_float2(bd.z, bd.w), make_float2(bd.x, bd.y)};
+                for (int it = 0; it < 2; ++it) fft_reg<R>(v[it]);
+                // output k2 is channel k1 + 128 + 16 k2 for k2 < 8 and k1 + 128 + 16 (k2 - 16) above
+                float2 r[2] = {make_float2(rr.x, rr.y), make_float2(rr.z, rr.w)};
+                float2 up[2] = {make_float2(ee.x, ee.y), make_float2(ee.z, ee.w)}, dn[2];
 #pragma unroll
-                for (int qq = 0; qq < 2; ++qq) {
-                    const int ku = k2 + qq, kd = R - 1 - ku;
+                for (int it = 0; it < 2; ++it) dn[it] = cmul(up[it], conj2(r[it]));
 #pragma unroll
-                    for (int it = 0; it < 2; ++it) {
-                        v[it][ku] = cmul(__fmul2_rn(v[it][ku], fu[qq]), up[it]);
-                        v[it][kd] = cmul(__fmul2_rn(v[it][kd], fd[qq]), dn[it]);
-                        up[it] = cmul(up[it], r[it]);
-                        dn[it] = cmul(dn[it], conj2(r[it]));
+                for (int k2 = 0; k2 < R / 2; k2 += 2) {
+                    const float4 bu = *reinterpret_cast<const float4 *>(bpt + k1 * R + k2);
+                    const float4 bd = *reinterpret_cast<const float4 *>(bpt + k1 * R + R - 2 - k2);
+                    const float2 fu[2] = {make_float2(bu.x, bu.y), make_float2(bu.z, bu.w)};
+                    const float2 fd[2] = {make_float2(bd.z, bd.w), make_float2(bd.x, bd.y)};
+#pragma unroll
+                    for (int qq = 0; qq < 2; ++qq) {
+                        const int ku = k2 + qq, kd = R - 1 - ku;
+#pragma unroll
+                        for (int it = 0; it < 2; ++it) {
+                            v[it][ku] = cmul(__fmul2_rn(v[it][ku], fu[qq]), up[it]);
+                            v[it][kd] = cmul(__fmul2_rn(v[it][kd], fd[qq]), dn[it]);
+                            up[it] = cmul(up[it], r[it]);
+                            dn[it] = cmul(dn[it], conj2(r[it]));
+                        }
                     }
                 }
             }
@@ -1007,11 +1063,11 @@ cudaError_t launch_t(const Handle &h, const void *raw, void *corr, const float *
         while (rpc > 1 && (long long)((rounds_total + rpc - 1) / rpc) * N * kPols * SB < 152LL * 4) rpc /= 2;
         dim3 grid(N * kPols, (rounds_total + rpc - 1) / rpc, SB);
         if (grid.y > 65535 || grid.z > 65535) return cudaErrorInvalidConfiguration;
-        constexpr size_t smem = ws256_smem_bytes<TIn>();
+        constexpr size_t smem = ws256_smem_bytes<TIn, OUT>();
         auto kern = ppf_correct_ws256_kernel<T, TIn, OUT>;
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        kern<<<grid, Ws256::ALL, smem, st>>>(reinterpret_cast<const TIn *>(raw), corr, h.d_taps, h.d_twiddle,
+        kern<<<grid, Ws256<OUT>::ALL, smem, st>>>(reinterpret_cast<const TIn *>(raw), corr, h.d_taps, h.d_twiddle,
                                                 h.d_phase, h.d_ratio, bandpass, gains, N, S, h.I_pad, s_out, scale, rpc, flags,
                                                 s_base, s_end, h.d_status, h.tc_timeout_cycles,
                                                 h.tc_test_no_tma);

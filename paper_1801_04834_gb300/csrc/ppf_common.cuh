@@ -83,7 +83,8 @@ enum {
     kBarFull = 3,    // FULL[0], FULL[1]: FIR round in the row buffer (ids 3, 4)
     kBarEmpty = 5,   // EMPTY[0], EMPTY[1]: FFT threads done with it (ids 5, 6)
     kBar256Full = 3,    // the 256-channel kernel's four row buffers: FULL (ids 3 to 6),
-    kBar256Empty = 7,   // EMPTY (ids 7 to 10)
+    kBar256Empty = 7,   // EMPTY (ids 7 to 10; with two buffers 7 and 8, and
+    kBar256EmptyF = 9,  // of the two tables of factors along time, ids 9 and 10)
     kBar256Fft = 11,    // each of its two FFT groups among itself (ids 11, 12)
 };
 __device__ __forceinline__ void named_bar_sync(int id, int n)
