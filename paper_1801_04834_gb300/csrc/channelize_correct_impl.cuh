@@ -29,11 +29,8 @@
 //                             so a warp store is one 256-byte run of the FP32
 //                             spectrum-blocked layout [SB][C][ceil16(S)/16][N][16][2]
 //                             or 2 inputs x 16 spectra of a planar plane;
-//   ppf_correct_ws256_kernel  C = 256, planar outputs: one CTA per (station,
-//                             pol), pass 2 with lane = spectrum;
-//   ppf_correct_kernel        C = 256, FP32 output: FIR and FFT alternating
-//                             on the same threads, writing from the pass-2
-//                             registers.
+//   ppf_correct_ws256_kernel  C = 256: one CTA per (station, pol), pass 2 with
+//                             a thread per two spectra.
 // Planar outputs are [SB][C][planes][I_pad][S_pad] (FP16/BF16 x operand_scale,
 // hi/lo FP16, or FP32 for the TF32-split X-stage); planar_pad zeroes what the
 // F-stage does not write (inputs I..I_pad, spectra past the last round).
@@ -50,19 +47,6 @@ namespace {
 using namespace ppf;
 
 // OUT: 1 FP32 spectrum-blocked, 2 FP16 planar, 3 BF16 planar, 4 split FP16 planar, 5 FP32 planar.
-// ppf_correct_kernel's per-round factor table: [kRound][IC inputs][PHC], rows
-// padded so that FFT pass 2 (lanes = 8 or 16 consecutive channels x inputs)
-// reads it conflict free
-template <int C>
-constexpr int fused_phc() { return C + (C == 16 ? 4 : 8); }
-
-template <int C, typename TIn>
-constexpr size_t fused_smem_bytes()
-{
-    using Cfg = PpfCfg<C>;
-    return ppf_smem_bytes<C, TIn>() + (size_t)kRound * Cfg::NPC * kPols * fused_phc<C>() * sizeof(float2);
-}
-
 // two values as 16-bit operands (OUT 3 BF16, else FP16), the first in the low half
 template <int OUT>
 __device__ __forceinline__ unsigned pack16(float a, float b)
@@ -102,203 +86,6 @@ __device__ __forceinline__ void store_planar(void *corr, long long o, long long 
             *reinterpret_cast<unsigned *>(out + 3 * pstride) = pack16_lo(ya.y, yb.y, im);
         }
     }
-}
-
-template <int C, int T, typename TIn, int OUT>
-__global__ void __launch_bounds__(PpfCfg<C>::NT, PpfCfg<C>::NT >= 512 ? 1 : 2)
-ppf_correct_kernel(const TIn *__restrict__ raw, void *__restrict__ corr, const float *__restrict__ taps,
-                   const float2 *__restrict__ twiddle, const float2 *__restrict__ phase,
-                   const float *__restrict__ bandpass, const float2 *__restrict__ gains, int N, int S, int I_pad,
-                   int S_pad, float scale, int rounds_per_cta, const float *__restrict__ flags, int s_base,
-                   int s_end)
-{
-    using Cfg = PpfCfg<C>;
-    constexpr int R = Cfg::R, NPC = Cfg::NPC, NT = Cfg::NT, ROW = Cfg::ROW;
-    constexpr int ROW_BYTES = C * kPols * (int)sizeof(TIn);
-    constexpr int BUF_BYTES = kRound * NPC * ROW_BYTES;
-    constexpr int IC = NPC * kPols;                 // inputs of this CTA
-    constexpr int PHC = fused_phc<C>();
-    constexpr int PHROW = IC * PHC;                 // factor-table row per spectrum
-    static_assert(OUT == 1, "FP32 spectrum-blocked output (planar outputs: the warp-specialised kernels)");
-    static_assert(NT >= 512 ? fused_smem_bytes<C, TIn>() <= 227 * 1024
-                            : 2 * (fused_smem_bytes<C, TIn>() + 1024) <= 228 * 1024,
-                  "two CTAs per SM (one at 512 threads)");
-    static_assert(ROW_BYTES % 16 == 0, "rows must be whole 16-byte chunks");
-
-    extern __shared__ __align__(16) unsigned char smem[];
-    float2 *tw = reinterpret_cast<float2 *>(smem);
-    unsigned char *inbuf = smem + C * sizeof(float2);
-    float2 *u = reinterpret_cast<float2 *>(inbuf + 2 * BUF_BYTES);
-    float2 *ph = u + Cfg::NTR * ROW;                // [kRound][IC][PHC] per-sample factors
-
-    const int tid = threadIdx.x;
-    const int sb = blockIdx.z;
-    const int n0 = blockIdx.x * NPC;                // station groups fastest
-    // spectra [s_base, s_end) of the block (s_base a multiple of 16); outputs are
-    // written at s - s_base with S_pad (planar) or S_pad (FP32: spectra per
-    // channel) as the output's spectrum stride
-    const int s0 = s_base + blockIdx.y * rounds_per_cta * kRound;
-    const int rows_total = S + T - 1;
-    const long long L = (long long)rows_total * C;
-    const int nrounds = min(rounds_per_cta, (s_end - s0 + kRound - 1) / kRound);
-    const int I = N * kPols;
-
-    auto stage = [&](int buf, int r0, int nrows) {
-        const int chunks = nrows * ROW_BYTES / 16;
-        for (int q = tid; q < NPC * chunks; q += NT) {
-            const int st = q / chunks, ch = q - st * chunks;
-            const int n = n0 + st;
-            const int row_in = (ch * 16) / ROW_BYTES;
-            const int byte_in_row = (ch * 16) - row_in * ROW_BYTES;
-            unsigned char *dst = inbuf + buf * BUF_BYTES + (row_in * NPC + st) * ROW_BYTES + byte_in_row;
-            const bool ok = (n < N) && (r0 + row_in < rows_total);
-            const unsigned char *src = reinterpret_cast<const unsigned char *>(raw);
-            if (ok) src += ((((long long)sb * N + n) * L + (long long)r0 * C) * kPols) * sizeof(TIn) + ch * 16;
-            cp_async16(dst, src, ok ? 16 : 0);
-        }
-    };
-
-    const int p = tid % kPols;
-    const int c = (tid / kPols) % C;
-    const int nl = tid / (kPols * C);
-
-    for (int i = tid; i < C; i += NT) tw[i] = twiddle[i];
-    // factor ownership: (station, channel) = tid mod NPC*C, spectra j = j0, j0+2, ...
-    constexpr int OWN = NPC * C;                    // = NT / 2
-    const int own_nc = tid % OWN, own_j0 = tid / OWN;
-    const int own_nl = own_nc / C, own_k = own_nc % C;
-    const int own_n = min(n0 + own_nl, N - 1);
-    const float2 pst = phase[((long long)sb * N + own_n) * C + own_k];   // (phi0, step)
-    float2 bgr[kPols];                              // bandpass x gain x scale of both pols
-#pragma unroll
-    for (int pp = 0; pp < kPols; ++pp) {
-        const float b = bandpass ? bandpass[(long long)own_n * C + own_k] : 1.f;
-        const float2 g = gains ? gains[own_n * kPols + pp] : make_float2(1.f, 0.f);
-        bgr[pp] = make_float2(b * g.x * scale, b * g.y * scale);
-    }
-
-    // taps duplicated into (h, h) pairs: one packed FMA filters re and im
-    float2 h[T];
-#pragma unroll
-    for (int k = 0; k < T; ++k) h[k] = make_float2(taps[k * C + c], taps[k * C + c]);
-
-    stage(1, s0, T - 1);
-    cp_async_commit();
-    stage(0, s0 + T - 1, kRound);
-    cp_async_commit();
-    cp_async_wait<1>();
-    __syncthreads();
-
-    float2 win[T];
-    const TIn *in1 = reinterpret_cast<const TIn *>(inbuf + BUF_BYTES);
-#pragma unroll
-    for (int k = 0; k < T - 1; ++k) win[k] = to_f2(in1[k * NT + tid]);
-    win[T - 1] = make_float2(0.f, 0.f);
-    __syncthreads();
-    if (nrounds > 1) stage(1, s0 + T - 1 + kRound, kRound);
-    cp_async_commit();
-
-    for (int b = 0; b < nrounds; ++b) {
-        const int sr = s0 + b * kRound;             // first spectrum of this round
-        cp_async_wait<1>();
-        __syncthreads();
-        // ---- FIR over 16 new rows ----
-        const TIn *in = reinterpret_cast<const TIn *>(inbuf + (b & 1) * BUF_BYTES);
-#pragma unroll
-        for (int j = 0; j < kRound; ++j) {
-            win[(T - 1 + j) % T] = to_f2(in[j * NT + tid]);
-            float2 acc = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int k = 0; k < T; ++k) {
-                acc = __ffma2_rn(h[k], win[(j + k) % T], acc);
-            }
-            u[(j * IC + nl * kPols + p) * ROW + c] = acc;
-        }
-        // ---- per-sample factors flag * bandpass * gain * exp(i phi) of this round ----
-#pragma unroll
-        for (int q = 0; q < kRound / 2; ++q) {
-            const int j = own_j0 + 2 * q;
-            const float phi = fmaf((float)(sr + j), pst.y, pst.x);
-            const float kq = rintf(phi * 0.15915494309189535f);           // phi / (2 pi)
-            float r = fmaf(-kq, 6.28125f, phi);                           // 2 pi = 6.28125 + 1.9353...e-3
-            r = fmaf(-kq, 1.9353071795864769e-3f, r);
-            float sn, cs;
-            __sincosf(r, &sn, &cs);
-            // lost-data weight of (station, spectrum); 1 without flags
-            const float fw = flags ? flags[(long long)own_n * S + min(sr + j, S - 1)] : 1.f;
-            cs *= fw;
-            sn *= fw;
-#pragma unroll
-            for (int pp = 0; pp < kPols; ++pp)
-                ph[j * PHROW + (own_nl * kPols + pp) * PHC + own_k] =
-                    make_float2(bgr[pp].x * cs - bgr[pp].y * sn, bgr[pp].x * sn + bgr[pp].y * cs);
-        }
-        __syncthreads();
-        if (b + 2 < nrounds) stage(b & 1, s0 + T - 1 + (b + 2) * kRound, kRound);
-        cp_async_commit();
-
-        // ---- FFT pass 1 (all inputs read before the transposed writes) ----
-        float2 y[Cfg::FFT_ITERS][R];
-#pragma unroll
-        for (int it = 0; it < Cfg::FFT_ITERS; ++it) {
-            const int task = it * NT + tid;
-            const float2 *row = u + (task / R) * ROW;
-#pragma unroll
-            for (int n1 = 0; n1 < R; ++n1) y[it][n1] = row[R * n1 + task % R];
-        }
-        __syncthreads();
-#pragma unroll
-        for (int it = 0; it < Cfg::FFT_ITERS; ++it) {
-            const int task = it * NT + tid;
-            const int tr = task / R, n2 = task % R;
-            float2 *row = u + tr * ROW;
-            fft_reg<R>(y[it]);
-#pragma unroll
-            for (int k1 = 1; k1 < R; ++k1) y[it][k1] = cmul(y[it][k1], tw[n2 * k1]);
-#pragma unroll
-            for (int k1 = 0; k1 < R; ++k1) row[(R + 1) * k1 + n2] = y[it][k1];
-        }
-        __syncthreads();
-        // ---- FFT pass 2 + correction, results held in registers ----
-#pragma unroll
-        for (int it = 0; it < Cfg::FFT_ITERS; ++it) {
-            const int task = it * NT + tid;
-            const int tr = task / R, k1 = task % R;  // transform tr = j * IC + il
-            const float2 *row = u + tr * ROW;
-#pragma unroll
-            for (int n2 = 0; n2 < R; ++n2) y[it][n2] = row[(R + 1) * k1 + n2];
-            fft_reg<R>(y[it]);
-            const int j = tr / IC, il = tr % IC;
-#pragma unroll
-            for (int k2 = 0; k2 < R; ++k2) {
-                const int kout = k1 + R * ((k2 + R / 2) % R);
-                y[it][k2] = cmul(y[it][k2], ph[j * PHROW + il * PHC + kout]);
-            }
-        }
-        {
-            // ---- write out from registers into the spectrum-blocked FP32 layout
-            // [SB][C][S_pad/16][N][16][2] (zeros past s_end) ----
-            float2 *out = reinterpret_cast<float2 *>(corr);
-            const int NB = S_pad / kRound;
-#pragma unroll
-            for (int it = 0; it < Cfg::FFT_ITERS; ++it) {
-                const int task = it * NT + tid;
-                const int tr = task / R, k1 = task % R;
-                const int s = sr + tr / IC, i = 2 * n0 + tr % IC;
-                if (i < I) {
-                    const int so = s - s_base;
-#pragma unroll
-                    for (int k2 = 0; k2 < R; ++k2) {
-                        const int kout = k1 + R * ((k2 + R / 2) % R);
-                        out[((((long long)sb * C + kout) * NB + so / kRound) * N + (i >> 1)) * (2 * kRound) +
-                            (so % kRound) * 2 + (i & 1)] = s < s_end ? y[it][k2] : make_float2(0.f, 0.f);
-                    }
-                }
-            }
-            // the next round's first barrier orders these reads of u before its FIR stores
-        }
-    }
-    cp_async_wait<0>();
 }
 
 // ---------------------------------------------------------------------------
@@ -357,7 +144,7 @@ constexpr int fused_ws_ctas()
 }
 
 
-// OUT as ppf_correct_kernel: 1 FP32 spectrum-blocked, 2 FP16 / 3 BF16 / 4 split
+// OUT: 1 FP32 spectrum-blocked, 2 FP16 / 3 BF16 / 4 split
 // FP16 / 5 FP32 planar ([SB][C][planes][I_pad][s_out], x scale for 2-4).
 template <int C, int T, typename TIn, int OUT>
 __global__ void __launch_bounds__(2 * FusedWsCfg<C>::NF, fused_ws_ctas<C, TIn>())
@@ -667,7 +454,7 @@ __global__ void __launch_bounds__(256) planar_pad_kernel(uint4 *__restrict__ cor
 }
 
 // ---------------------------------------------------------------------------
-// Warp-specialised fused kernel for C = 256 with planar outputs (OUT = 2..5):
+// Warp-specialised fused kernel for C = 256:
 // one CTA per (station, pol) and SM, 256 FIR threads (one channel each) and 256
 // FFT threads in two groups of 128. A round's rows (16 spectra of one input) fit
 // twice in shared memory at this channel count only per input; the CTAs of a
@@ -707,12 +494,14 @@ __global__ void __launch_bounds__(256) planar_pad_kernel(uint4 *__restrict__ cor
 //    store on distinct banks).
 // 64 stations, 61 subbands of int8, 768 spectra, before this form -> now: FP32
 // planes 4.44 -> 4.13 ms (3.7 TB/s of raw rows and operands), FP16 4.45 -> 4.38
-// ms. With
+// ms,
+// spectrum-blocked FP32 10.97 -> 5.07 ms (FIR and FFT alternating on the same
+// threads of a CTA for both pols). With
 // anchors, two row buffers instead of four took 4.34 for 4.16 ms, four FIR
 // outputs at a time instead of eight 4.16 for 4.01.
 template <int OUT>
 struct Ws256 {
-    static constexpr bool TIME = OUT <= 3;              // factors along time (16-bit operands)
+    static constexpr bool TIME = OUT == 2 || OUT == 3;              // factors along time (16-bit operands)
     static constexpr int C = 256, R = 16;
     static constexpr int NF = C, NG = 128;              // FIR threads; FFT threads of a group
     static constexpr int ALL = NF + 2 * NG;
@@ -752,7 +541,6 @@ ppf_correct_ws256_kernel(const TIn *__restrict__ raw, void *__restrict__ corr, c
     constexpr int BUF_BYTES = kRound * ROW_BYTES;
     constexpr int NG = W::NG;
     constexpr int HAND = NF + NG;               // FULL / EMPTY: the FIR threads and one FFT group
-    static_assert(OUT >= 2 && OUT <= 5, "planar outputs");
     static_assert(ROW_BYTES % 16 == 0, "rows must be whole 16-byte chunks");
     static_assert(ws256_smem_bytes<TIn, OUT>() <= 227 * 1024, "one CTA per SM");
 
@@ -996,11 +784,33 @@ ppf_correct_ws256_kernel(const TIn *__restrict__ raw, void *__restrict__ corr, c
                     if (s + 1 >= s_end) v[1][k2] = make_float2(0.f, 0.f);
                 }
             }
-            const long long base = (long long)sb * C * planes * pstride + (long long)i * s_out + (s - s_base);
+            if constexpr (OUT == 1) {
+                // Spectrum-blocked: the 16 spectra of a channel are every other 8 bytes
+                // of a 256-byte run (the other pol's CTA fills the rest in L2). The
+                // lanes of an even and of the next odd k1 swap a spectrum each, so a
+                // store holds all 16 spectra of one channel, both values of each sector
+                // at once.
+                const bool odd = k1 & 1;
+                const long long kstride = (long long)(s_out / kRound) * N * (2 * kRound);
+                float2 *out = reinterpret_cast<float2 *>(corr) +
+                              ((long long)sb * C + (k1 & ~1)) * kstride +
+                              ((long long)((sr - s_base) / kRound) * N + n) * (2 * kRound) + (jp + odd) * 2 + p;
 #pragma unroll
-            for (int k2 = 0; k2 < R; ++k2) {
-                const int kout = k1 + R * ((k2 + R / 2) % R);
-                store_planar<OUT>(corr, base + (long long)kout * planes * pstride, pstride, v[0][k2], v[1][k2]);
+                for (int k2 = 0; k2 < R; ++k2) {
+                    const float2 mine = odd ? v[1][k2] : v[0][k2], give = odd ? v[0][k2] : v[1][k2];
+                    const float2 got = make_float2(__shfl_xor_sync(0xffffffffu, give.x, 8),
+                                                   __shfl_xor_sync(0xffffffffu, give.y, 8));
+                    float2 *o = out + (long long)(R * ((k2 + R / 2) % R)) * kstride;
+                    o[0] = odd ? got : mine;
+                    o[kstride] = odd ? mine : got;
+                }
+            } else {
+                const long long base = (long long)sb * C * planes * pstride + (long long)i * s_out + (s - s_base);
+#pragma unroll
+                for (int k2 = 0; k2 < R; ++k2) {
+                    const int kout = k1 + R * ((k2 + R / 2) % R);
+                    store_planar<OUT>(corr, base + (long long)kout * planes * pstride, pstride, v[0][k2], v[1][k2]);
+                }
             }
         }
     }
@@ -1025,7 +835,6 @@ template <int C, int T, typename TIn, int OUT>
 cudaError_t launch_t(const Handle &h, const void *raw, void *corr, const float *bandpass, const float2 *gains,
                      const float *flags, const FWindow *win, cudaStream_t st)
 {
-    using Cfg = PpfCfg<C>;
     const int N = h.p.n_stations, S = h.p.n_spectra, SB = h.p.n_subbands;
     // spectra [s_base, s_end) into an output whose spectrum stride is s_out
     const int s_base = win ? win->s_base : 0;
@@ -1056,7 +865,8 @@ cudaError_t launch_t(const Handle &h, const void *raw, void *corr, const float *
         e = cudaGetLastError();
         if (e != cudaSuccess || OUT == 1) return e;
         return planar_pad(h, corr, OUT, rounds_total * kRound, s_out, st);
-    } else if constexpr (C == 256 && OUT != 1) {
+    } else {
+        static_assert(C == 256, "16, 64 or 256 channels");
         // one CTA per (station, pol) and SM; long runs of rounds amortise the
         // prologue, shortened only while the grid would be under ~4 waves
         int rpc = 64;
@@ -1071,23 +881,6 @@ cudaError_t launch_t(const Handle &h, const void *raw, void *corr, const float *
                                                 h.d_phase, h.d_ratio, bandpass, gains, N, S, h.I_pad, s_out, scale, rpc, flags,
                                                 s_base, s_end, h.d_status, h.tc_timeout_cycles,
                                                 h.tc_test_no_tma);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        return planar_pad(h, corr, OUT, rounds_total * kRound, s_out, st);
-    } else {
-        const int sgroups = (N + Cfg::NPC - 1) / Cfg::NPC;
-        // long runs of rounds per CTA amortise the T-1 history rows each CTA reads
-        // and filters first; shorten them only while the grid would be under ~8 waves
-        int rpc = 32;
-        while (rpc > 1 && (long long)((rounds_total + rpc - 1) / rpc) * sgroups * SB < 152LL * 16) rpc /= 2;
-        dim3 grid(sgroups, (rounds_total + rpc - 1) / rpc, SB);
-        if (grid.y > 65535 || grid.z > 65535) return cudaErrorInvalidConfiguration;
-        constexpr size_t smem = fused_smem_bytes<C, TIn>();
-        auto kern = ppf_correct_kernel<C, T, TIn, OUT>;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        kern<<<grid, Cfg::NT, smem, st>>>(reinterpret_cast<const TIn *>(raw), corr, h.d_taps, h.d_twiddle, h.d_phase,
-                                          bandpass, gains, N, S, h.I_pad, s_out, scale, rpc, flags, s_base, s_end);
         e = cudaGetLastError();
         if (e != cudaSuccess || OUT == 1) return e;
         return planar_pad(h, corr, OUT, rounds_total * kRound, s_out, st);

@@ -170,7 +170,7 @@ extern "C" fx_status fx_create(const fx_params *pp, fx_handle **out)
     FX_TRY(cudaMalloc(&h->d_twiddle, sizeof(float2) * C));
     FX_TRY(cudaMalloc(&h->d_centres, sizeof(double) * SB));
     FX_TRY(cudaMalloc(&h->d_phase, sizeof(float2) * SB * N * C));
-    if (C == 256 && (p.precision == FX_TF32_SPLIT || p.precision == FX_F16_SPLIT))
+    if (C == 256 && p.precision != FX_F16 && p.precision != FX_BF16)
         FX_TRY(cudaMalloc(&h->d_ratio, sizeof(float2) * N * (size_t)((S + 15) / 16 * 16)));
     FX_TRY(cudaMalloc(&h->d_status, sizeof(int) * 4));
     FX_TRY(cudaMalloc(&h->d_xf32_tiles, sizeof(int2) * ntiles));

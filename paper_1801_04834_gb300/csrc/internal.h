@@ -23,7 +23,7 @@ struct Handle {
     float2 *d_twiddle = nullptr;       // [C]  exp(-2 pi i m / C), from host FP64
     double *d_centres = nullptr;       // [SB]
     float2 *d_phase = nullptr;         // [SB][N][C] (phi0 mod 2pi, per-spectrum step)
-    float2 *d_ratio = nullptr;         // C = 256, FP32 or split FP16 planes: [N][ceil16(S)] exp(2 pi i (fs / 16) tau_n(s))
+    float2 *d_ratio = nullptr;         // C = 256, not FP16/BF16: [N][ceil16(S)] exp(2 pi i (fs / 16) tau_n(s))
     int *d_status = nullptr;           // device-side error word
     int2 *d_xf32_tiles = nullptr;      // tile list of the FP32 correlator
     int xf32_ntiles = 0;

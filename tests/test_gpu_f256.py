@@ -55,3 +55,31 @@ def test_factors_against_fp64(N, SB, S, tau, fmt):
     assert rel(out) < 1.5 * rel(two) + 2.3e-6, (rel(out), rel(two))
     assert torch.all(out[:, :, :, :, S:] == 0) and torch.all(out[:, :, :, c.I:] == 0)
     c.close()
+
+
+@pytest.mark.parametrize("N,SB,S,tau", [(3, 2, 16, 5e-6), (2, 1, 83, 1e-4), (5, 1, 200, 2e-3), (1, 3, 1, 0.0)])
+@pytest.mark.parametrize("fmt", [synth.CI16, synth.CI8])
+def test_spectrum_blocked_factors_against_fp64(N, SB, S, tau, fmt):
+    """The same factors and bound for FX_F32, whose stores swap spectra between lanes."""
+    import paper_1801_04834_gb300 as m
+    from paper_1801_04834_gb300.api import f32_unblock
+    rng = np.random.default_rng(S)
+    blk = synth.make_block(9 + S, fmt, SB, N, 256, S, sigma=100.0 if fmt == synth.CI16 else 20.0)
+    c = m.Correlator(N, SB, 256, S, taps=blk.taps, centres=blk.centres, n_taps=16, fmt=fmt)
+    d0 = torch.from_numpy(rng.uniform(-tau, tau, N)).cuda()
+    d1 = d0 + torch.from_numpy(rng.uniform(-tau, tau, N)).cuda() / 10
+    bp = torch.from_numpy(rng.uniform(0.5, 1.5, (N, 256)).astype(np.float32)).cuda()
+    g = torch.from_numpy(synth.random_gains(rng, N).astype(np.float32)).cuda()
+    raw = torch.from_numpy(blk.raw).cuda()
+    out = torch.full(c.corr_shape(), float("nan"), device="cuda")
+    c.channelize_correct(raw, d0, d1, bandpass=bp, gains=g, out=out)
+    chan = c.channelize(raw)
+    two = c.correct(chan, d0, d1, bandpass=bp, gains=g)
+    ref = corrected64(c, chan, blk.centres, d0, d1, bp, g)
+
+    def rel(t):
+        y = f32_unblock(t, S).double().reshape(SB, 256, S, c.I, 2).permute(0, 1, 4, 3, 2)
+        return ((y - ref).norm() / ref.norm()).item()
+    assert rel(out) < 1.5 * rel(two) + 2.3e-6, (rel(out), rel(two))
+    assert torch.all(f32_unblock(out, out.shape[2] * 16)[:, :, S:] == 0)
+    c.close()
