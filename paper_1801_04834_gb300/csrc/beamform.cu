@@ -109,8 +109,8 @@ __device__ __forceinline__ unsigned short weight_bits(float x, unsigned bf16)
 
 // Weight table W[sb][k][3][NB_pad][64], planes (im, re, -im): one thread per
 // (subband, beam, station slot), looping over channels. Padding is zero.
-// One thread writes two neighbouring stations' weights of one beam over a
-// quarter of the channels, so a warp's store is a whole 128-byte row. Bound by
+// One thread writes two neighbouring stations' weights of one beam over all
+// channels (or a quarter of them), so a warp's store is a whole 128-byte row. Bound by
 // the table's bytes (40 subbands x 256 channels x 128 beams, 503 MB: 137 us;
 // one station per thread, 2-byte stores, 171 us).
 __global__ void __launch_bounds__(256)
@@ -608,7 +608,11 @@ cudaError_t launch_beamform(const Handle &h, const void *corr, int NB, const dou
 
     // weight table for this call
     const long long wthreads = (long long)SB * NB_pad * 32;
-    bf_weight_kernel<<<dim3((unsigned)((wthreads + 255) / 256), 4), 256, 0, st>>>(
+    // channels split four ways where a thread's FP64 set-up is small beside them, or
+    // where the blocks would not fill the SMs (7 stations, 16 beams, 64 channels, one
+    // subband: the whole beam call 73 us unsplit)
+    const unsigned wblocks = (unsigned)((wthreads + 255) / 256);
+    bf_weight_kernel<<<dim3(wblocks, C >= 256 || wblocks < 152 ? 4 : 1), 256, 0, st>>>(
         delays, weights, h.d_centres, h.d_bfw, SB, C, N, NB, NB_pad, h.p.sample_rate_hz, bf16);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
