@@ -109,44 +109,56 @@ __device__ __forceinline__ unsigned short weight_bits(float x, unsigned bf16)
 
 // Weight table W[sb][k][3][NB_pad][64], planes (im, re, -im): one thread per
 // (subband, beam, station slot), looping over channels. Padding is zero.
-// One thread writes two neighbouring stations' weights of one beam over all
-// channels (or a quarter of them), so a warp's store is a whole 128-byte row. Bound by
-// the table's bytes (40 subbands x 256 channels x 128 beams, 503 MB: 137 us;
-// one station per thread, 2-byte stores, 171 us).
+// A thread sets up one station of one beam in FP64, neighbouring lanes swap what
+// they have set up, and each writes both stations' weights for every other
+// channel (of all, or of a part of them), so stores are whole 64-byte runs. Bound
+// by the table's bytes at many channels (40 subbands x 256 channels x 128 beams,
+// 503 MB: 171 us with one station per thread and 2-byte stores, 137 with two), by
+// the set-up at few.
 __global__ void __launch_bounds__(256)
 bf_weight_kernel(const double *__restrict__ delays, const float *__restrict__ weights,
                  const double *__restrict__ centres, unsigned short *__restrict__ W, int SB, int C, int N, int NB,
                  int NB_pad, double fs, unsigned bf16)
 {
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long long)SB * NB_pad * 32) return;
-    const int n = 2 * (int)(idx % 32);
-    const int b = (int)((idx / 32) % NB_pad);
-    const int sb = (int)(idx / (32LL * NB_pad));
+    if (idx >= (long long)SB * NB_pad * 64) return;        // whole warps
+    const int n0 = (int)(idx % 64), odd = n0 & 1, n = n0 - odd;
+    const int b = (int)((idx / 64) % NB_pad);
+    const int sb = (int)(idx / (64LL * NB_pad));
     const long long plane = (long long)NB_pad * 64;
-    const int kq4 = (C + gridDim.y - 1) / gridDim.y, kb = blockIdx.y * kq4, ke = min(C, kb + kq4);
+    const int part = (C + gridDim.y - 1) / gridDim.y, kb = blockIdx.y * part + odd, ke = min(C, kb - odd + part);
     unsigned *w = reinterpret_cast<unsigned *>(W + ((long long)sb * C + kb) * 3 * plane + (long long)b * 64 + n);
     const long long step = plane / 2;
-    if (b >= NB || n >= N) {
-        for (int k = kb; k < ke; ++k, w += 3 * step) w[0] = w[step] = w[2 * step] = 0;
+    if (b >= NB) {                                         // the same for a whole warp
+        for (int k = kb; k < ke; k += 2, w += 6 * step) w[0] = w[step] = w[2 * step] = 0;
         return;
     }
     const double two_pi = 6.283185307179586476925286766559;
     float p0f[2], dpf[2], a[2];
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-        const bool in = n + q < N;
-        const double d = in ? delays[(long long)b * N + n + q] : 0.0;
+    {
+        const bool in = n0 < N;
+        const double d = in ? delays[(long long)b * N + n0] : 0.0;
         // phase at channel 0 (frequency centre - fs/2) and step per channel (fs / C), mod 2 pi
         double p0 = two_pi * (centres[sb] - 0.5 * fs) * d;
         p0 -= two_pi * rint(p0 / two_pi);
         double dp = two_pi * (fs / C) * d;
         dp -= two_pi * rint(dp / two_pi);
-        a[q] = in ? (weights ? weights[n + q] : 1.f) : 0.f;
-        p0f[q] = (float)p0;
-        dpf[q] = (float)dp;
+        const float own[3] = {(float)p0, (float)dp, in ? (weights ? weights[n0] : 1.f) : 0.f};
+        float both[3][2];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const float other = __shfl_xor_sync(0xffffffffu, own[q], 1);
+            both[q][0] = odd ? other : own[q];
+            both[q][1] = odd ? own[q] : other;
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            p0f[q] = both[0][q];
+            dpf[q] = both[1][q];
+            a[q] = both[2][q];
+        }
     }
-    for (int k = kb; k < ke; ++k, w += 3 * step) {
+    for (int k = kb; k < ke; k += 2, w += 6 * step) {
         unsigned j = 0, re = 0, mj = 0;
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
@@ -607,12 +619,12 @@ cudaError_t launch_beamform(const Handle &h, const void *corr, int NB, const dou
     if (planes / 2 * 3 > 0x7fffffffLL) return cudaErrorInvalidValue;
 
     // weight table for this call
-    const long long wthreads = (long long)SB * NB_pad * 32;
-    // channels split four ways where a thread's FP64 set-up is small beside them, or
-    // where the blocks would not fill the SMs (7 stations, 16 beams, 64 channels, one
-    // subband: the whole beam call 73 us unsplit)
+    const long long wthreads = (long long)SB * NB_pad * 64;
+    // channels split where a thread's FP64 set-up is small beside them, or where the
+    // blocks would not fill the SMs (7 stations, 16 beams, 64 channels, one subband:
+    // the whole beam call 73 us unsplit, 62 in four)
     const unsigned wblocks = (unsigned)((wthreads + 255) / 256);
-    bf_weight_kernel<<<dim3(wblocks, C >= 256 || wblocks < 152 ? 4 : 1), 256, 0, st>>>(
+    bf_weight_kernel<<<dim3(wblocks, wblocks < 152 ? 4 : C >= 256 ? 2 : 1), 256, 0, st>>>(
         delays, weights, h.d_centres, h.d_bfw, SB, C, N, NB, NB_pad, h.p.sample_rate_hz, bf16);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
