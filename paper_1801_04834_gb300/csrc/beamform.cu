@@ -129,7 +129,7 @@ bf_weight_kernel(const double *__restrict__ delays, const float *__restrict__ we
     const int part = (C + gridDim.y - 1) / gridDim.y, kb = blockIdx.y * part + odd, ke = min(C, kb - odd + part);
     unsigned *w = reinterpret_cast<unsigned *>(W + ((long long)sb * C + kb) * 3 * plane + (long long)b * 64 + n);
     const long long step = plane / 2;
-    if (b >= NB) {                                         // the same for a whole warp
+    if (b >= NB || (n0 & ~31) >= N) {                     // the same for a whole warp
         for (int k = kb; k < ke; k += 2, w += 6 * step) w[0] = w[step] = w[2 * step] = 0;
         return;
     }
