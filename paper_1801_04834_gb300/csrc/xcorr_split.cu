@@ -436,6 +436,15 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_split_kernel(const __grid
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
+    if constexpr (BLOCKED) {
+        // Station slots that no copy fills (the padding of I_pad, a last tile's absent
+        // channels) are converted with the rest of their warp, and the largest value
+        // there chooses how the real stations are split: they start as zeros, not as
+        // what an earlier kernel left in shared memory.
+        for (unsigned q = threadIdx.x; q < (unsigned)P.lands * P.land_bytes / 16; q += kT3Threads)
+            reinterpret_cast<uint4 *>(land)[q] = make_uint4(0, 0, 0, 0);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
     if (warp == kT3MmaWarp) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                      "r"(kT3TmemCols)
