@@ -1,20 +1,27 @@
 // xcorr_split.cu -- FP32-accurate X-stage on the tcgen05 tensor cores, any
 // station count: FP32 corrected samples split in the kernel into hi + lo,
-// V ~ hi hi' + hi lo' + lo hi' (lo lo' dropped), the main term hi hi' as TF32
-// MMAs and the cross terms as BF16 MMAs, FP32 accumulation in TMEM, chunk
+// V ~ hi hi' + hi lo' + lo hi' (lo lo' dropped), FP32 accumulation in TMEM, chunk
 // sums added in IEEE FP32 in registers. Serves FX_TF32_SPLIT (planar FP32
-// operands) and FX_F32 (spectrum-blocked complex operands).
+// operands; hi hi' as TF32 MMAs, the cross terms as BF16 MMAs) and FX_F32
+// (spectrum-blocked complex operands; every term as TF32 MMAs).
 //
 // Paper, Sec. "Signal processing with GPU kernels": the correlator forms
 // V[a][b] = sum_s Y[s][a] conj(Y[s][b]) for all input pairs and integrates over
 // the block, in single precision. TF32 keeps FP32's exponent range with an
-// 11-bit significand; hi = x with its 13 low mantissa bits cleared is exactly
-// a TF32 value and lo = x - hi is exact in FP32 with |lo| < 2^-10 |x|. The
-// cross terms hi lo' and lo hi' are each below 2^-10 of the product, so they
-// tolerate BF16 operands: rounding hi and lo to BF16 (8-bit significand, FP32
-// exponent range, round to nearest) changes a cross term by at most 2^-8 of
-// itself, i.e. 2^-18 of the product in the worst case and about 2^-21 RMS,
-// with zero mean; the dropped lo lo' term is below 2^-20 of the product.
+// 11-bit significand.
+//   FX_TF32_SPLIT: hi = x with its 13 low mantissa bits cleared is exactly a TF32
+// value and lo = x - hi is exact in FP32 with |lo| < 2^-10 |x|. The cross terms
+// hi lo' and lo hi' are each below 2^-10 of the product; rounding hi and lo to
+// BF16 (8-bit significand, FP32 exponent range, round to nearest) changes one by
+// at most 2^-8 of itself, i.e. 2^-18 of the product in the worst case and about
+// 2^-21 RMS, with zero mean; the dropped lo lo' term is below 2^-20 of the product.
+//   FX_F32 takes the place of an FP32 FMA chain and may lose no more than that
+// does. hi is x rounded to TF32, so |lo| <= 2^-11 |x| with both signs; a TF32 MMA
+// reads 11 of lo's at most 12 bits (2^-24 of x RMS), and lo lo' is 2^-24 of the
+// product RMS. With BF16 cross terms, as above, the error of one product, 2^-21, showed
+// wherever a chain is short or its sum small: uncorrelated stations up to 768
+// spectra (2.3 times the chain's at 128) and lossy blocks (half of the spectra
+// lost: 4.6 times at 128, 1.9 at 768).
 //
 // What bounds it: shared-memory bandwidth (tensor-core operand reads plus the
 // converter's traffic), then the tensor pipe. So a diagonal tile, where row
@@ -27,22 +34,24 @@
 // cross term appears once instead of with its conjugate). Per stage of 16
 // spectra and n = 128 inputs:
 //   TF32 (K = 8, two K-steps): hJ x [hR; hJ] (N = 2n), hR x hR (N = n)
-//   BF16 (K = 16):             hJ x [lR; 2lJ], hR x [-lJ; 2lR] (N = 2n)
-// into one accumulator of 2n columns [Q | P]: 640 tensor clocks and 64 KB of
-// operand reads, against 1024 clocks and 96 KB with all products formed, and
-// 24 KB of converter stores against 32 KB. 64 stations x 1280 channels x 3072
+//   BF16 (K = 16) or TF32:     hJ x [lR; 2lJ], hR x [-lJ; 2lR] (N = 2n)
+// into one accumulator of 2n columns [Q | P]: with BF16 cross terms 640 tensor
+// clocks and 64 KB of operand reads, against 1024 clocks and 96 KB with all
+// products formed, and 24 KB of converter stores against 32 KB; with TF32 ones
+// 896 clocks, 88 KB and 48 KB. 64 stations x 1280 channels x 3072
 // spectra (4.0 GB of operands): planar 1.45 ms with every product formed and
 // the chunk sums reduced in L2, 0.98 ms so (4.1 TB/s; without its MMAs the
-// kernel takes 0.66 ms, without its converter 0.95 ms); blocked 1.26 ms,
-// against 6.09 ms on the CUDA cores.
+// kernel takes 0.66 ms, without its converter 0.95 ms); blocked 1.31 ms with
+// chains of 32 spectra (1.22 with 64, 1.63 with 16; BF16 cross terms 1.27 with
+// 64), against 6.09 ms on the CUDA cores.
 //
 // Work items. Rows come in blocks of 128 inputs (M = 128); an item is
 // (subband x channel, row block, column block) over the upper block
 // triangle: the diagonal item of a row block covers columns
 // [row0, row0 + min(128, I_pad - row0)), off-diagonal items cover the columns
 // right of it in tiles of at most 64 inputs and form every product:
-//   TF32: hJ_a x [hR; hJ], hR_a x [-hJ; hR]
-//   BF16: hJ_a x [lR; lJ], hR_a x [-lJ; lR], lJ_a x [hR; hJ], lR_a x [-hJ; hR]
+//   TF32:         hJ_a x [hR; hJ], hR_a x [-hJ; hR]
+//   BF16 or TF32: hJ_a x [lR; lJ], hR_a x [-lJ; lR], lJ_a x [hR; hJ], lR_a x [-hJ; hR]
 // with Q = Im V and P = Re V. 64 stations (128 inputs) is one diagonal item
 // per channel; 76 stations (160 inputs) is a 128-column diagonal item, a
 // 32-column off-diagonal item and a 32-row diagonal item.
@@ -57,16 +66,24 @@
 //             non-zero low bits check this against an FP64 reference).
 //   blocked   one station's 16 spectra x 2 pols are 256 contiguous bytes; a
 //             stage lands by one bulk copy, and the converter writes hi rounded
-//             to TF32 (which halves lo) as 64-byte rows, 64-byte swizzle.
+//             to TF32 (which halves lo) and lo as 64-byte rows, 64-byte swizzle.
 // Planes of n rows each:
-//   diagonal item:     TF32 R, J; BF16 hR, hJ, lR, 2lJ, -lJ, 2lR. The A operands
-//                      are planes R, J, hR, hJ read as 128-row tiles: rows past n
-//                      are other planes' data and only reach accumulator rows
-//                      that are not used; the regions are large enough that
-//                      these reads stay inside.
-//   off-diagonal item: 128-row planes TF32 R, J, BF16 hR, hJ, lR, lJ of the row
-//                      inputs; TF32 -J, R, J, BF16 -hJ, hR, hJ, -lJ, lR, lJ of
-//                      the columns.
+//   diagonal item:     planar TF32 R, J; BF16 hR, hJ, lR, 2lJ, -lJ, 2lR; blocked
+//                      those six in FP32. The A operands are planes R, J, hR, hJ
+//                      read as 128-row tiles: rows past n are other planes' data
+//                      and only reach accumulator rows that are not used; the
+//                      regions are large enough that these reads stay inside.
+//   off-diagonal item: planar 128-row planes TF32 R, J, BF16 hR, hJ, lR, lJ of the
+//                      row inputs; TF32 -J, R, J, BF16 -hJ, hR, hJ, -lJ, lR, lJ
+//                      of the columns; blocked hR, hJ, lR, lJ of the rows, then
+//                      -hJ, hR, hJ, -lJ, lR, lJ of the columns.
+//
+// An infinity (blocked). Its hi is the infinity, which meets the other station's
+// hi and lo: with a lo of 0 or of the other sign the sum of the two products
+// would be a NaN where the product is an infinity; and so it would where both
+// overflow. So the converter warps of a stage vote, and if one has met an infinity
+// or a value of 2^64 or more all convert the stage again with truncated hi and
+// a lo of x's sign that is never zero (split1, SAFE).
 //
 // Accumulation. The tensor core's FP32 accumulator does not round each
 // addition to nearest, so a long chain of MMAs into one accumulator drifts
@@ -74,8 +91,8 @@
 // every `chunk` stages and the chunk sums are added in registers (round to
 // nearest): the eight epilogue warps hold the whole 128 x 256 accumulator, 128
 // registers per thread, so nothing is read back or reduced in memory until
-// the item ends. 64 spectra per chunk for FX_TF32_SPLIT; 16 for FX_F32, whose
-// reference is the rounding of an FP32 FMA chain (measured in
+// the item ends. 64 spectra per chunk for FX_TF32_SPLIT; 16 or 32 for FX_F32,
+// whose reference is the rounding of an FP32 FMA chain (measured in
 // xf32_on_tensor_cores). Each visibility is summed by one lane in a fixed
 // order, so results are reproducible.
 //
@@ -124,9 +141,12 @@ constexpr int kT3MaxStages = 6;
 constexpr int kT3MaxItems = 64;                       // items per channel
 constexpr int kT3TmemCols = 512;
 constexpr int kT3AccCols = 256;
-constexpr int kT3Bars = 4 * kT3MaxStages + 6;         // full, conv, empty, landed per stage; accf 2, acce 2, exch, drain
+// full, conv, empty, landed per stage; accf 2, acce 2, exch, drain, vote per converter group
+constexpr int kT3Bars = 4 * kT3MaxStages + 6 + kT3ConvGroups;
+constexpr unsigned kT3Ctrl = 8u * kT3Bars + 16u + 8u * kT3ConvGroups;   // barriers, TMEM base, abort flag, votes
 constexpr int kT3Blk = 32 * 33;                       // one 32 x 32 block of the transpose scratch, padded rows
 constexpr unsigned kT3Scratch = 10u * kT3Blk * 4u;    // lower block triangle of a 128 x 128 plane
+constexpr unsigned kT3ScratchMid = 8u * kT3Blk * 4u;  // six blocks at a time, or the blocks of four segments of 32 inputs
 constexpr unsigned kT3ScratchSmall = 4u * kT3Blk * 4u; // four blocks at a time
 constexpr unsigned kT3SmemMax = 227u * 1024u;
 
@@ -152,7 +172,7 @@ struct T3Params {
     int stages, lands;        // depth of the operand ring and of the landing ring
     unsigned stage_bytes, land_bytes;
     unsigned row_land;        // blocked: offset of the row inputs' stations in a landing slot
-    unsigned scratch_bytes;   // kT3Scratch or kT3ScratchSmall
+    unsigned scratch_bytes;   // kT3Scratch, kT3ScratchMid or kT3ScratchSmall
     int no_tma;               // failure-detection test hook: issue no loads
     int accumulate;           // add to vis
 };
@@ -238,52 +258,52 @@ __device__ __forceinline__ uint2 dbl_bf16x4(uint2 v)   // exact: doubling only m
     return make_uint2(*reinterpret_cast<unsigned *>(&a), *reinterpret_cast<unsigned *>(&b));
 }
 
-// One value's hi part (a TF32 value) and, through *lo, x - hi.
+// One value's hi part (a TF32 value) and, through *lo, x - hi (exact).
 //  TRUNC  the 13 low bits cleared: what a TF32 MMA reads of the raw value
 //  ROUND  rounded to nearest: lo is half as large and has both signs
-//  SAFE   as TRUNC, and an infinity has no low part (inf - inf would turn its
-//         products into NaN); for the values ROUND could carry to infinity
+//  SAFE   as TRUNC, for stages that hold an infinity or a value whose products may
+//         overflow: lo has x's sign and is never zero, so that an infinity times
+//         the other station's hi and lo is the same infinity twice, not a NaN
 enum SplitMode { TRUNC, ROUND, SAFE };
 template <int MODE>
 __device__ __forceinline__ float split1(float x, float *lo)
 {
     const unsigned b = __float_as_uint(x);
     const float h = __uint_as_float((MODE == ROUND ? b + 0x1000u : b) & 0xFFFFE000u);
-    *lo = MODE == SAFE && fabsf(x) == __int_as_float(0x7f800000) ? 0.f : x - h;
+    *lo = x - h;
+    if (MODE == SAFE && x == x && !(fabsf(*lo) > 0.f)) *lo = copysignf(1.17549435e-38f, x);
     return h;
 }
-constexpr unsigned kT3RoundMax = 0x7f7f0000u;          // FP32 bits from which SAFE is taken, below
-constexpr unsigned kT3BfMax = 0x7f7f8000u;             // those that round to infinity in BF16
+constexpr float kT3RoundMax = 0x1p64f;                 // from here on SAFE: hi lo' may overflow
 
-// hi and lo parts of four FP32 values: hi in FP32, both in BF16 (round to nearest even)
-struct Split4 {
-    float4 hf;
-    uint2 h, l;
-};
 template <int MODE>
-__device__ __forceinline__ Split4 split4(float4 x)
+__device__ __forceinline__ void split4(float4 x, float4 &h, float4 &l)
 {
-    Split4 r;
-    float4 l;
-    r.hf.x = split1<MODE>(x.x, &l.x);
-    r.hf.y = split1<MODE>(x.y, &l.y);
-    r.hf.z = split1<MODE>(x.z, &l.z);
-    r.hf.w = split1<MODE>(x.w, &l.w);
-    // SAFE: what BF16 would round to infinity takes no part in the cross terms, whose
-    // signs are not the product's (inf - inf); the main term carries the infinity
-    auto b = [](float h) { return MODE == SAFE && fabsf(h) >= __uint_as_float(kT3BfMax) ? 0.f : h; };
-    r.h = make_uint2(bf16x2(b(r.hf.x), b(r.hf.y)), bf16x2(b(r.hf.z), b(r.hf.w)));
-    r.l = make_uint2(bf16x2(l.x, l.y), bf16x2(l.z, l.w));
-    return r;
+    h.x = split1<MODE>(x.x, &l.x);
+    h.y = split1<MODE>(x.y, &l.y);
+    h.z = split1<MODE>(x.z, &l.z);
+    h.w = split1<MODE>(x.w, &l.w);
 }
 
-// Operand planes: DIAG column planes of a diagonal item (BF16 hR, hJ, lR, 2lJ,
-// -lJ, 2lR), COLS column planes of an off-diagonal item (BF16 -hJ, hR, hJ, -lJ,
-// lR, lJ; a TF32 plane -J before R and J), ROWS row planes of an off-diagonal
-// item (BF16 hR, hJ, lR, lJ).
+// hi and lo of four values of the planar layout, in BF16 (round to nearest even)
+struct SplitBf4 {
+    uint2 h, l;
+};
+__device__ __forceinline__ SplitBf4 split_bf4(float4 x)
+{
+    float4 h, l;
+    split4<TRUNC>(x, h, l);
+    return {make_uint2(bf16x2(h.x, h.y), bf16x2(h.z, h.w)), make_uint2(bf16x2(l.x, l.y), bf16x2(l.z, l.w))};
+}
+
+// Operand planes: DIAG column planes of a diagonal item (hR, hJ, lR, 2lJ, -lJ,
+// 2lR), COLS column planes of an off-diagonal item (-hJ, hR, hJ, -lJ, lR, lJ),
+// ROWS row planes of an off-diagonal item (hR, hJ, lR, lJ). In BF16 beside the
+// landed TF32 rows (planar; a TF32 plane -J before R and J for COLS), or all in
+// FP32 (blocked).
 enum PlaneRole { DIAG, COLS, ROWS };
 template <int ROLE>
-__device__ __forceinline__ void put_bf(const Split4 &a, const Split4 &b, unsigned char *bf, unsigned bp)
+__device__ __forceinline__ void put_bf(const SplitBf4 &a, const SplitBf4 &b, unsigned char *bf, unsigned bp)
 {
     auto put = [&](int plane, uint2 v) { *reinterpret_cast<uint2 *>(bf + plane * bp) = v; };
     if constexpr (ROLE == DIAG) {
@@ -309,6 +329,33 @@ __device__ __forceinline__ void put_bf(const Split4 &a, const Split4 &b, unsigne
 }
 
 __device__ __forceinline__ float4 neg4(float4 v) { return make_float4(-v.x, -v.y, -v.z, -v.w); }
+__device__ __forceinline__ float4 dbl4(float4 v) { return make_float4(v.x + v.x, v.y + v.y, v.z + v.z, v.w + v.w); }
+
+template <int ROLE>
+__device__ __forceinline__ void put_tf(float4 hr, float4 hj, float4 lr, float4 lj, unsigned char *tf, unsigned tp)
+{
+    auto put = [&](int plane, float4 v) { *reinterpret_cast<float4 *>(tf + plane * tp) = v; };
+    if constexpr (ROLE == DIAG) {
+        put(0, hr);
+        put(1, hj);
+        put(2, lr);
+        put(3, dbl4(lj));
+        put(4, neg4(lj));
+        put(5, dbl4(lr));
+    } else if constexpr (ROLE == COLS) {
+        put(0, neg4(hj));
+        put(1, hr);
+        put(2, hj);
+        put(3, neg4(lj));
+        put(4, lr);
+        put(5, lj);
+    } else {
+        put(0, hr);
+        put(1, hj);
+        put(2, lr);
+        put(3, lj);
+    }
+}
 
 // Planar operands: the R and J planes (128-byte rows of 32 spectra, 128-byte
 // swizzle, pitch tp) at tf hold the raw rows; this is their half `half`. A
@@ -326,24 +373,25 @@ __device__ __forceinline__ void convert_planar(unsigned char *tf, unsigned tp, u
         const float4 x = *reinterpret_cast<const float4 *>(p);
         const float4 y = *reinterpret_cast<const float4 *>(p + tp);
         if constexpr (ROLE == COLS) *reinterpret_cast<float4 *>(p - tp) = neg4(y);
-        put_bf<ROLE>(split4<TRUNC>(x), split4<TRUNC>(y), bf + r8 * 256 + bo, bp);
+        put_bf<ROLE>(split_bf4(x), split_bf4(y), bf + r8 * 256 + bo, bp);
     }
 }
 
 // Spectrum-blocked operands: `land` holds stations' runs of [16 spectra][2
 // pols] complex values; a task is 4 spectra of one station, both pols, written
-// to the TF32 planes (64-byte rows, 64-byte swizzle, pitch tp) too. Spectra from
+// to the FP32 planes (64-byte rows, 64-byte swizzle, pitch tp). Spectra from
 // s_lim on count as zero (every gst stations seg fewer: time segments). The four 16-byte reads of a task are rotated by
 // lane / 2 so that eight lanes' reads fall on distinct banks, and sorted again
 // in registers. Rows are ordered pol by pol within eight stations (row 16 (st /
 // 8) + 8 p + st mod 8), so that the lanes of a store take consecutive rows and
-// distinct banks too.
-template <int ROLE, bool SEG>
-__device__ __forceinline__ void convert_blocked(const unsigned char *land, unsigned char *tf, unsigned tp,
-                                                unsigned char *bf, unsigned bp, int rows, int s_lim, int gst, int seg, int t)
+// distinct banks too. Returns whether a value of this thread's wants SAFE.
+template <int ROLE, bool SEG, int MODE>
+__device__ __forceinline__ bool convert_blocked(const unsigned char *land, unsigned char *tf, unsigned tp, int rows,
+                                                int s_lim, int gst, int seg, int t)
 {
     const int nt = rows / 2 * 4;                          // a multiple of 32: whole warps
     const int rot = (t >> 1) & 3;
+    float top = 0.f;
     for (int q = t; q < nt; q += 32 * kT3ConvWarps) {
         const float4 *w = reinterpret_cast<const float4 *>(land) + 4 * q;
         float4 v[4], u[4];
@@ -360,30 +408,20 @@ __device__ __forceinline__ void convert_blocked(const unsigned char *land, unsig
             for (int e = 0; e < 4; ++e)
                 if (4 * lc + e >= lim) v[e] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        float top = 0.f;
+        if constexpr (MODE == ROUND) {
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-            top = fmaxf(fmaxf(fmaxf(top, fabsf(v[e].x)), fabsf(v[e].y)), fmaxf(fabsf(v[e].z), fabsf(v[e].w)));
-        const bool safe = __any_sync(0xffffffffu, top >= __uint_as_float(kT3RoundMax));
-        auto put = [&](auto mode) {
-            constexpr int MODE = decltype(mode)::value;
+            for (int e = 0; e < 4; ++e)
+                top = fmaxf(fmaxf(fmaxf(top, fabsf(v[e].x)), fabsf(v[e].y)), fmaxf(fabsf(v[e].z), fabsf(v[e].w)));
+        }
 #pragma unroll
-            for (int p = 0; p < kPols; ++p) {
-                const int r = 16 * (st >> 3) + 8 * p + (st & 7);
-                const Split4 x = split4<MODE>(p ? make_float4(v[0].z, v[1].z, v[2].z, v[3].z)
-                                                : make_float4(v[0].x, v[1].x, v[2].x, v[3].x));
-                const Split4 y = split4<MODE>(p ? make_float4(v[0].w, v[1].w, v[2].w, v[3].w)
-                                                : make_float4(v[0].y, v[1].y, v[2].y, v[3].y));
-                unsigned char *o = tf + tf_off(r, lc);
-                *reinterpret_cast<float4 *>(o) = x.hf;
-                *reinterpret_cast<float4 *>(o + tp) = y.hf;
-                if constexpr (ROLE == COLS) *reinterpret_cast<float4 *>(o - tp) = neg4(y.hf);
-                put_bf<ROLE>(x, y, bf + bf_off(r, lc), bp);
-            }
-        };
-        if (safe) put(std::integral_constant<int, SAFE>{});
-        else put(std::integral_constant<int, ROUND>{});
+        for (int p = 0; p < kPols; ++p) {
+            float4 hr, hj, lr, lj;
+            split4<MODE>(p ? make_float4(v[0].z, v[1].z, v[2].z, v[3].z) : make_float4(v[0].x, v[1].x, v[2].x, v[3].x), hr, lr);
+            split4<MODE>(p ? make_float4(v[0].w, v[1].w, v[2].w, v[3].w) : make_float4(v[0].y, v[1].y, v[2].y, v[3].y), hj, lj);
+            put_tf<ROLE>(hr, hj, lr, lj, tf + tf_off(16 * (st >> 3) + 8 * p + (st & 7), lc), tp);
+        }
     }
+    return top >= kT3RoundMax;
 }
 
 // BLOCKED: spectrum-blocked complex operands (FX_F32), else planar (FX_TF32_SPLIT)
@@ -409,8 +447,10 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_split_kernel(const __grid
     auto acce_bar = [&](int b) { return bar0 + 8u * (4 * kT3MaxStages + 2 + b); };
     const unsigned exch_bar = bar0 + 8u * (4 * kT3MaxStages + 4);
     const unsigned drain_bar = bar0 + 8u * (4 * kT3MaxStages + 5);
+    auto vote_bar = [&](int g) { return bar0 + 8u * (4 * kT3MaxStages + 6 + g); };  // a converter group's warps have voted
     unsigned *tmem_slot = reinterpret_cast<unsigned *>(ctrl + 8 * kT3Bars);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
+    volatile unsigned *votes = tmem_slot + 2;          // [group][parity]: the last stage that needs SAFE
     // TF32 operands: blocked, planes of 64-byte rows in the stage; planar, planes
     // of 128-byte rows (32 spectra) in the landing slot
     constexpr unsigned TROW = BLOCKED ? 64u : 128u;
@@ -432,6 +472,10 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_split_kernel(const __grid
         }
         mbar_init(exch_bar, kT3EpiWarps);
         mbar_init(drain_bar, 1);
+        for (int g = 0; g < kT3ConvGroups; ++g) {
+            mbar_init(vote_bar(g), kT3ConvWarps);
+            votes[2 * g] = votes[2 * g + 1] = 0;
+        }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -564,8 +608,7 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_split_kernel(const __grid
                     const bool diag = itm.w != 0;
                     // plane pitches and the offset of the column BF16 planes, in 16-byte units
                     const unsigned tp = (unsigned)n * TROW / 16, bp = (unsigned)n * kT3BfRow / 16;
-                    const unsigned bf0 = BLOCKED ? (diag ? 2 * tp : (2 * TA + 4 * kT3ABf) / 16 + 3 * tp)
-                                                 : (diag ? 0u : 4 * kT3ABf / 16);
+                    const unsigned bf0 = diag ? 0u : 4 * kT3ABf / 16;
                     const unsigned id2 = idesc_tf32(2 * n), id1 = idesc_tf32(n);
                     const unsigned idb = make_idesc(1u, 2 * n, false);
                     for (int k0 = 0; k0 < P.nk && ok; k0 += P.chunk, ++acc_it) {
@@ -589,11 +632,19 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_split_kernel(const __grid
                             const unsigned long long tf =
                                 tdesc0 + (BLOCKED ? so : (unsigned)l * (P.land_bytes >> 4) + 4u * ((k0 + kc) % PER));
                             const unsigned long long bf = bdesc0 + so + bf0;
+                            // (the small cross terms first, while the accumulator is small: 10 to 20% less
+                            // error than after the main term)
                             if (diag) {
-                                // (the small cross terms first, while the accumulator is small: 10% less
-                                // error than after the main term)
-                                mma_f16(d, bf + bp, bf + 2 * bp, idb, kc ? 1u : 0u);                 // hJ x [lR; 2lJ]
-                                mma_f16(d, bf, bf + 4 * bp, idb, 1u);                                // hR x [-lJ; 2lR]
+                                if constexpr (BLOCKED) {
+#pragma unroll
+                                    for (int kk = 0; kk < kT3K / 8; ++kk) {
+                                        mma_tf32(d, tf + tp + 2u * kk, tf + 2 * tp + 2u * kk, id2, (kc | kk) ? 1u : 0u);   // hJ x [lR; 2lJ]
+                                        mma_tf32(d, tf + 2u * kk, tf + 4 * tp + 2u * kk, id2, 1u);                         // hR x [-lJ; 2lR]
+                                    }
+                                } else {
+                                    mma_f16(d, bf + bp, bf + 2 * bp, idb, kc ? 1u : 0u);             // hJ x [lR; 2lJ]
+                                    mma_f16(d, bf, bf + 4 * bp, idb, 1u);                            // hR x [-lJ; 2lR]
+                                }
 #pragma unroll
                                 for (int kk = 0; kk < kT3K / 8; ++kk)      // 8 FP32 = 32 bytes per TF32 K-step
                                     mma_tf32(d, tf + tp + 2u * kk, tf + 2u * kk, id2, 1u);           // hJ x [hR; hJ]
@@ -601,14 +652,27 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_split_kernel(const __grid
                                 for (int kk = 0; kk < kT3K / 8; ++kk)
                                     mma_tf32(d + (unsigned)n, tf + 2u * kk, tf + 2u * kk, id1, 1u);  // hR x hR
                             } else {
-                                // rows: TF32 R, J, BF16 hR, hJ, lR, lJ; columns: TF32 -J, R, J, BF16 -hJ, hR, hJ, -lJ, lR, lJ
-                                const unsigned long long ra = bdesc0 + so + (BLOCKED ? 2 * TA / 16 : 0u);
-                                const unsigned long long tb = tf + (BLOCKED ? 2 * TA + 4 * kT3ABf : 2 * TA) / 16;
-                                constexpr unsigned AP = kT3ABf / 16;
-                                mma_f16(d, ra + AP, bf + 4 * bp, idb, kc ? 1u : 0u);  // hJ x [lR; lJ]
-                                mma_f16(d, ra, bf + 3 * bp, idb, 1u);                 // hR x [-lJ; lR]
-                                mma_f16(d, ra + 3 * AP, bf + bp, idb, 1u);            // lJ x [hR; hJ]
-                                mma_f16(d, ra + 2 * AP, bf, idb, 1u);                 // lR x [-hJ; hR]
+                                // rows: R, J, lR, lJ; columns: -J, R, J, -lJ, lR, lJ (planar: the lo planes and
+                                // the cross terms' hi planes in BF16)
+                                const unsigned long long tb = tf + (BLOCKED ? 4 * TA : 2 * TA) / 16;
+                                if constexpr (BLOCKED) {
+                                    constexpr unsigned AP = TA / 16;
+#pragma unroll
+                                    for (int kk = 0; kk < kT3K / 8; ++kk) {
+                                        const unsigned long long ra = tf + 2u * kk, cb = tb + 2u * kk;
+                                        mma_tf32(d, ra + AP, cb + 4 * tp, id2, (kc | kk) ? 1u : 0u);   // hJ x [lR; lJ]
+                                        mma_tf32(d, ra, cb + 3 * tp, id2, 1u);                         // hR x [-lJ; lR]
+                                        mma_tf32(d, ra + 3 * AP, cb + tp, id2, 1u);                    // lJ x [hR; hJ]
+                                        mma_tf32(d, ra + 2 * AP, cb, id2, 1u);                         // lR x [-hJ; hR]
+                                    }
+                                } else {
+                                    const unsigned long long ra = bdesc0 + so;
+                                    constexpr unsigned AP = kT3ABf / 16;
+                                    mma_f16(d, ra + AP, bf + 4 * bp, idb, kc ? 1u : 0u);  // hJ x [lR; lJ]
+                                    mma_f16(d, ra, bf + 3 * bp, idb, 1u);                 // hR x [-lJ; lR]
+                                    mma_f16(d, ra + 3 * AP, bf + bp, idb, 1u);            // lJ x [hR; hJ]
+                                    mma_f16(d, ra + 2 * AP, bf, idb, 1u);                 // lR x [-hJ; hR]
+                                }
 #pragma unroll
                                 for (int kk = 0; kk < kT3K / 8; ++kk) {
                                     mma_tf32(d, tf + TA / 16 + 2u * kk, tb + tp + 2u * kk, id2, 1u);   // hJ x [hR; hJ]
@@ -637,6 +701,7 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_split_kernel(const __grid
             const int grp = (warp - kT3ConvWarp0) / kT3ConvWarps, cw = (warp - kT3ConvWarp0) % kT3ConvWarps;
             const int ct = cw * 32 + lane;
             Ring ring, lring;
+            unsigned voted = 0;                         // blocked: stages this group has voted on
             int turn = 0;                               // group of the next stage
             bool ok = true;
             for (long long w = blockIdx.x; w < P.n_items && ok; w += gridDim.x) {
@@ -666,13 +731,26 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_split_kernel(const __grid
                     unsigned char *la = land + (size_t)l * P.land_bytes;
                     if constexpr (BLOCKED) {
                         const int lim = P.S - kc * kT3K, gst = P.gin / 2, seg = P.nk * kT3K;
-                        if (diag) {
-                            convert_blocked<DIAG, SEG>(la, st, pitch, st + 2 * pitch, bpitch, n, lim, gst, seg, ct);
-                        } else {
-                            unsigned char *tb = st + 2 * TA + 4 * kT3ABf;
-                            convert_blocked<ROWS, false>(la + P.row_land, st, TA, st + 2 * TA, kT3ABf, 128, lim, gst, seg, ct);
-                            convert_blocked<COLS, false>(la, tb + pitch, pitch, tb + 3 * pitch, bpitch, n, lim, gst, seg, ct);
+                        auto convert = [&](auto mode) {
+                            constexpr int MODE = decltype(mode)::value;
+                            if (diag) return convert_blocked<DIAG, SEG, MODE>(la, st, pitch, n, lim, gst, seg, ct);
+                            const bool rows = convert_blocked<ROWS, false, MODE>(la + P.row_land, st, TA, 128, lim, gst, seg, ct);
+                            return convert_blocked<COLS, false, MODE>(la, st + 4 * TA, pitch, n, lim, gst, seg, ct) || rows;
+                        };
+                        // An infinity meets every other station's lo parts, which other warps of the
+                        // group may have written: they all have to know of it. (Bounded like every
+                        // wait here, hence no named barrier: a warp may have left on an abort.)
+                        const bool big = __any_sync(0xffffffffu, convert(std::integral_constant<int, ROUND>{}));
+                        ++voted;
+                        volatile unsigned *vote = votes + 2 * grp + (voted & 1u);
+                        if (big) *vote = voted;
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(vote_bar(grp));
+                        if (!__all_sync(0xffffffffu, t3wait(vote_bar(grp), (voted & 1u) ^ 1u, abort_flag, P, 4))) {
+                            ok = false;
+                            break;
                         }
+                        if (*vote == voted) convert(std::integral_constant<int, SAFE>{});
                     } else {
                         const int half = kc % PER;
                         if (diag) {
@@ -748,17 +826,15 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_split_kernel(const __grid
                 // Re V = (P + P') / 2, Im V = Q - Q': each warp puts its 32 x 32 blocks
                 // on or below the diagonal into the scratch and reads the mirror
                 // blocks of those on or above it (rows of 33 words: no bank
-                // conflicts), all ten blocks at once or, with the small scratch, in
-                // three phases of three, three and the four diagonal ones
-                const bool small = P.scratch_bytes < kT3Scratch;
+                // conflicts), all ten blocks at once or, with less scratch, the diagonal
+                // ones last, after six others at once or three and three. Channels or
+                // segments of up to 32 inputs need the diagonal blocks only.
+                const bool small = P.gin <= 32;
+                const int phases = small || P.scratch_bytes >= kT3Scratch ? 1 : P.scratch_bytes >= kT3ScratchMid ? 2 : 3;
                 auto place = [&](int r, int c, int &slot) {     // block (r, c), c <= r: phase and slot
-                    if (!small) {
-                        slot = r * (r + 1) / 2 + c;
-                        return 0;
-                    }
-                    const int o = r * (r - 1) / 2 + c;
-                    slot = r == c ? r : o % 3;
-                    return r == c ? 2 : o / 3;
+                    const int o = r * (r - 1) / 2 + c;          // rank among those below the diagonal
+                    slot = r == c ? r : phases == 1 ? 4 + o : phases == 2 ? o : o % 3;
+                    return r == c ? phases - 1 : small ? -1 : phases == 3 ? o / 3 : 0;
                 };
                 auto put = [&](const float2 (&A)[32], int phase) {
 #pragma unroll
@@ -791,14 +867,14 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_split_kernel(const __grid
                         }
                     }
                 };
-                for (int ph = 0; ph < (small ? 3 : 1) && live; ++ph) {
+                for (int ph = 0; ph < phases && live; ++ph) {
                     put(V, ph);
                     live = sync8();
                     if (!live) break;
                     take(V, ph, 0.5f, 0.5f);
                     live = sync8();
                 }
-                for (int ph = 0; ph < (small ? 3 : 1) && live; ++ph) {
+                for (int ph = 0; ph < phases && live; ++ph) {
                     put(Q, ph);
                     live = sync8();
                     if (!live) break;
@@ -920,8 +996,8 @@ int t3_group(int I_pad, long long channels, int num_sms)
 // no room in the tile, or in the scratch for the blocks.
 int t3_segments(int I_pad, int group, int nk)
 {
-    static_assert(2u * 2u * 48u * 48u * 4u <= kT3Scratch && 2u * 4u * 32u * 32u * 4u <= kT3Scratch,
-                  "the segments' blocks fit the scratch");
+    static_assert(2u * 2u * 48u * 48u * 4u <= kT3Scratch && 2u * 4u * 32u * 32u * 4u <= kT3ScratchMid,
+                  "the segments' blocks fit the scratch (two of 48 inputs leave the tile below 128)");
     return group > 1 || I_pad > 48 ? 1 : std::max(1, std::min(128 / I_pad, nk / 4));
 }
 
@@ -936,34 +1012,34 @@ bool t3_plan(int I_pad, bool blocked, int side, T3Plan &pl)
 {
     constexpr int NT = 64;                              // columns of an off-diagonal item
     pl.items.clear();
-    unsigned nmax = 0;                                  // widest off-diagonal item
+    unsigned nmax = 0, ndmax = 0;                       // widest off-diagonal and diagonal item
     const unsigned trow = blocked ? 64u : 128u;         // bytes of a TF32 row; planar: in the landing slot
     unsigned tf = 0, bf = 0;
     for (int row0 = 0; row0 < I_pad; row0 += 128) {
         const unsigned nd = (unsigned)std::min(128, I_pad - row0) * side;
         pl.items.push_back(make_int4(row0, row0, (int)nd, 1));
         // the planes, and the 128-row reads of the A operands J (TF32) and hJ (BF16)
-        tf = std::max(tf, std::max(2u * nd, nd + 128u) * trow);
+        tf = std::max(tf, std::max((blocked ? 6u : 2u) * nd, nd + 128u) * trow);
         bf = std::max(bf, std::max(6u * nd, nd + 128u) * kT3BfRow);
+        ndmax = std::max(ndmax, nd);
         for (int c0 = row0 + 128; c0 < I_pad; c0 += NT) {
             const int n = std::min(NT, I_pad - c0);
             pl.items.push_back(make_int4(row0, c0, n, 0));
             nmax = std::max(nmax, (unsigned)n);
-            tf = std::max(tf, (256u + 3u * n) * trow);
+            tf = std::max(tf, (blocked ? 512u + 6u * n : 256u + 3u * n) * trow);
             bf = std::max(bf, (512u + 6u * n) * kT3BfRow);
         }
     }
     if ((int)pl.items.size() > kT3MaxItems) return false;
-    // (blocked: both regions in one stage, BF16 planes right after that item's TF32
-    // planes, so a diagonal item's need is below the sum too)
     const unsigned k1 = 1023u;
-    pl.stage_bytes = ((blocked ? tf + bf : bf) + k1) & ~k1;
+    pl.stage_bytes = ((blocked ? tf : bf) + k1) & ~k1;
     pl.land_bytes = ((blocked ? (64u + nmax / 2) * kT3StRun : tf) + k1) & ~k1;
     pl.row_land = nmax / 2 * kT3StRun;
     // off-diagonal items have larger stages: the small scratch makes room for a third
-    // of them up to 80 stations (78 stations x 1024 channels x 1001 spectra: 873 -> 779 us)
-    pl.scratch_bytes = nmax ? kT3ScratchSmall : kT3Scratch;
-    const unsigned room = kT3SmemMax - 1024u - pl.scratch_bytes - 8u * kT3Bars - 16u;
+    // of them up to 80 stations (planar, 78 stations x 1024 channels x 1001 spectra: 873 -> 779 us)
+    // and so does the middle one beside full blocked tiles
+    pl.scratch_bytes = nmax ? kT3ScratchSmall : blocked && ndmax == 128u ? kT3ScratchMid : kT3Scratch;
+    const unsigned room = kT3SmemMax - 1024u - pl.scratch_bytes - kT3Ctrl;
     pl.stages = std::min<int>(kT3MaxStages - 1, (int)(room / (pl.stage_bytes + pl.land_bytes)));
     // blocked slots hold one stage: one more of them where it fits
     pl.lands = pl.stages + (blocked && (pl.stages + 1) * pl.land_bytes + pl.stages * pl.stage_bytes <= room ? 1 : 0);
@@ -1027,7 +1103,7 @@ cudaError_t t3_launch(const Handle &h, const void *corr, float2 *vis, cudaStream
     P.no_tma = h.tc_test_no_tma;
     P.accumulate = accumulate ? 1 : 0;
     const size_t smem = 1024 + (size_t)pl.stages * pl.stage_bytes + (size_t)pl.lands * pl.land_bytes + pl.scratch_bytes +
-                        8 * kT3Bars + 16;
+                        kT3Ctrl;
     auto kern = segs > 1 ? xcorr_split_kernel<BLOCKED, true> : xcorr_split_kernel<BLOCKED, false>;
     // the register split draws on what the launch brings: refuse a build with less
     cudaFuncAttributes fa;
@@ -1056,14 +1132,19 @@ cudaError_t launch_xcorr_split(const Handle &h, const float *corr, float2 *vis, 
 }
 
 // FX_F32 goes to the tensor cores where that is at least as accurate as the
-// CUDA-core FMA chain, whose error grows with its length: against FP64 on
-// noise with a common signal (normwise, 2 to 130 stations) the chain has
-// 2.4e-7 at 128 spectra, 3.2e-7 at 256, 4.2e-7 at 384, 6.4e-7 at 1024, 8.5e-7 at
-// 1536, 1.2e-6 at 3072; the split has 1.6e-7 to 2.4e-7 from 128 spectra on with
-// accumulator chains of 16 spectra, 2.5e-7 to 3.3e-7 with 32 and 4.8e-7 to
-// 6.9e-7 with 64. Longer chains drain less often (64 stations x 1280 channels
-// x 3072 spectra: 1.53 ms with 16, 1.26 ms with 64; CUDA cores 6.09 ms), so the
-// longest that stays below the FMA chain is taken. Shorter integrations and the
+// CUDA-core FMA chain, whose error grows with its length. Against FP64, over all
+// baselines normwise / over the cross baselines, error as a multiple of the
+// chain's (8, 50 and 76 stations; the chain has 2.4e-7 at 128 spectra, 4e-7 at 384,
+// 6e-7 at 768, 1.2e-6 at 3072):
+//   spectra (accumulator chain)    128 (16)    384 (16)    768 (16)    1024 (32)   3072 (32)
+//   uncorrelated noise            0.74 0.46   0.46 0.30   0.35 0.24   0.56 0.37   0.37 0.24
+//   with a common signal          0.65 0.44   0.37 0.27   0.26 0.21   0.49 0.39   0.26 0.23
+//   half of the spectra lost      0.86 0.80   0.59 0.54   0.44 0.44   0.63 0.56   0.43 0.37
+// Chains of 32 would have up to 1.7 at 128 spectra and 1.2 at 384 (half lost); they drain
+// the accumulator half as often (64 stations x 1280 channels x 1024 spectra 476 us,
+// with 16 583, CUDA cores 2056). What the chain length cannot mend is a baseline
+// with few live spectra, where an FMA chain barely rounds: 64 live spectra 0.9 0.8
+// of its error, 16 1.2 1.2, 4 2.1 2.0, one 3.4 3.3 (1e-7 of the product). Shorter integrations and the
 // forms asked for by flag stay on the CUDA cores.
 constexpr int kXf32TcSpectra = 128;
 
@@ -1076,8 +1157,7 @@ bool xf32_on_tensor_cores(const Handle &h)
 
 cudaError_t launch_xcorr_f32_tc(const Handle &h, const float2 *corr, float2 *vis, cudaStream_t st, bool accumulate)
 {
-    const int S = h.p.n_spectra;
-    return t3_launch<true>(h, corr, vis, st, accumulate, S >= 1536 ? 4 : S >= 384 ? 2 : 1);
+    return t3_launch<true>(h, corr, vis, st, accumulate, h.p.n_spectra >= 1024 ? 2 : 1);
 }
 
 }  // namespace fxi
