@@ -706,8 +706,8 @@ def run_fx(args, w):
     return 0
 
 
-# X-stage forms timed beside the headline: (precision, FP32 form); "2x4" is the CUDA-core X-stage
-VARIANTS = ((4, "auto"), (0, "auto"), (0, "2x4"), (1, "auto"), (2, "auto"), (3, "auto"))
+# X-stage forms timed beside the headline: (precision, FP32 form); "4x4" is the CUDA-core X-stage
+VARIANTS = ((4, "auto"), (0, "auto"), (0, "4x4"), (1, "auto"), (2, "auto"), (3, "auto"))
 
 
 def variant_name(vp, form):

@@ -127,13 +127,15 @@ typedef struct {
 #define FX_FLAG_STREAMING 0x1u
 
 /* Forms of the FP32 X-stage (results agree up to FP32 rounding). Default: the
- * tensor cores from 128 spectra on (fx_correlate), else the CUDA cores with
- * 4 x 4-station register tiles from 16 stations up (2 x 4 below). SMALL: the
- * CUDA cores with 2 x 4 tiles. THREE_MULT: the same with the
- * three-multiplication complex product (sum xr yr, sum xi yi,
- * sum (xr + xi)(yr - yi)): 3 FMAs per complex MAC instead of 4. */
+ * tensor cores from 128 spectra on (fx_correlate), else the CUDA cores.
+ * CUDA_CORES: FP32 FMAs on those for any number of spectra, with 4 x 4-station
+ * register tiles from 16 stations up (2 x 4 below). SMALL: the same with 2 x 4
+ * tiles always. THREE_MULT: 2 x 4 tiles with the three-multiplication complex
+ * product (sum xr yr, sum xi yi, sum (xr + xi)(yr - yi)): 3 FMAs per complex
+ * MAC instead of 4. At most one of the three. */
 #define FX_FLAG_XF32_SMALL_TILES 0x2u
 #define FX_FLAG_XF32_THREE_MULT 0x4u
+#define FX_FLAG_XF32_CUDA_CORES 0x10u
 
 /* Failure-detection test hook: the tensor-core X-stage issues no operand
  * loads, so its consumer waits run out after about a millisecond; the call

@@ -84,9 +84,11 @@ class Correlator:
         p.h_subband_centre_hz = centres.ctypes.data_as(ctypes.POINTER(ctypes.c_double))
         p.h_taps = taps.ctypes.data_as(ctypes.POINTER(ctypes.c_float))
         p.operand_scale = operand_scale
-        # FP32 X-stage form: "auto" (tensor cores from 128 spectra on), or on the CUDA cores
-        # "2x4" tiles or "3mult" (2x4 tiles with the three-multiplication complex product)
-        form = {"auto": 0, "2x4": _abi.FX_FLAG_XF32_SMALL_TILES, "3mult": _abi.FX_FLAG_XF32_THREE_MULT}[xf32_form]
+        # FP32 X-stage form: "auto" (tensor cores from 128 spectra on), or FP32 FMAs on the CUDA
+        # cores in "4x4" tiles (from 16 stations up), "2x4" tiles, or "3mult" (2x4 tiles with the
+        # three-multiplication complex product)
+        form = {"auto": 0, "4x4": _abi.FX_FLAG_XF32_CUDA_CORES, "2x4": _abi.FX_FLAG_XF32_SMALL_TILES,
+                "3mult": _abi.FX_FLAG_XF32_THREE_MULT}[xf32_form]
         p.flags = (_abi.FX_FLAG_STREAMING if streaming else 0) | form | extra_flags
         p.host_chunk_subbands = host_chunk_subbands
         p.max_coarse_shift = max_coarse_shift

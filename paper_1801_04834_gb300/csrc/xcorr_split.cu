@@ -1151,7 +1151,7 @@ constexpr int kXf32TcSpectra = 128;
 bool xf32_on_tensor_cores(const Handle &h)
 {
     T3Plan pl;
-    return (h.p.flags & (FX_FLAG_XF32_SMALL_TILES | FX_FLAG_XF32_THREE_MULT)) == 0 &&
+    return (h.p.flags & (FX_FLAG_XF32_CUDA_CORES | FX_FLAG_XF32_SMALL_TILES | FX_FLAG_XF32_THREE_MULT)) == 0 &&
            h.p.n_spectra >= kXf32TcSpectra && t3_plan(h.I_pad, true, 1, pl);
 }
 

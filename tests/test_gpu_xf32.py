@@ -122,3 +122,21 @@ def test_infinities_as_on_the_cuda_cores(N, S):
     assert torch.equal(torch.isposinf(a), torch.isposinf(b)) and torch.equal(torch.isneginf(a), torch.isneginf(b))
     plain = [k for k in range(C) if k % 3 != 1 or k > 10]
     assert torch.equal(a[:, plain], b[:, plain])      # sums of whole numbers below 2^24: exact in both
+
+
+@pytest.mark.parametrize("N,S", [(5, 300), (20, 1100), (64, 128)])
+def test_cuda_core_form_at_any_length(N, S):
+    """The FP32 FMA chain in 4 x 4 tiles (2 x 4 below 16 stations), also where the tensor cores
+    are the default: per visibility the same chain as in 2 x 4 tiles, bit for bit."""
+    import paper_1801_04834_gb300 as m
+    C = 16
+    y = operands("noise", N, C, S)
+    corr, vis = m.f32_block(y), {}
+    for form in ("4x4", "2x4", "auto"):
+        c = correlator(N, 1, C, S, xf32_form=form)
+        vis[form] = c.correlate(corr)
+        c.close()
+    assert torch.equal(vis["4x4"], vis["2x4"])
+    assert not torch.equal(vis["4x4"], vis["auto"])   # the default is another form at this length
+    ref = product(y)
+    assert ((vis["4x4"].double() - ref).norm() / ref.norm()).item() < S * 2.0 ** -24
