@@ -471,7 +471,7 @@ __global__ void __launch_bounds__(256) planar_pad_kernel(uint4 *__restrict__ cor
 //  * FP32 and split FP16: the phase factors come from the channel axis. f_k is
 //    linear in k, so for a spectrum s exp(i phi(k, s)) = e(k1, s) r(s)^m for
 //    k = k1 + 128 + 16 m: the FIR threads put one anchor e (16 x 16 per round,
-//    each the gain, flag and scale times one __sincosf) into a table, the
+//    each the gain, flag and scale times one sine and cosine) into a table, the
 //    phase-table kernel has left r(s) = exp(2 pi i (fs / 16) tau(s)) per station
 //    and spectrum, and an FFT thread steps from its anchor up and down eight
 //    channels each in registers.
@@ -495,7 +495,7 @@ __global__ void __launch_bounds__(256) planar_pad_kernel(uint4 *__restrict__ cor
 // 64 stations, 61 subbands of int8, 768 spectra, before this form -> now: FP32
 // planes 4.44 -> 4.13 ms (3.7 TB/s of raw rows and operands), FP16 4.45 -> 4.38
 // ms,
-// spectrum-blocked FP32 10.97 -> 5.07 ms (FIR and FFT alternating on the same
+// spectrum-blocked FP32 10.97 -> 4.86 ms (FIR and FFT alternating on the same
 // threads of a CTA for both pols). With
 // anchors, two row buffers instead of four took 4.34 for 4.16 ms, four FIR
 // outputs at a time instead of eight 4.16 for 4.01.
@@ -616,14 +616,19 @@ ppf_correct_ws256_kernel(const TIn *__restrict__ raw, void *__restrict__ corr, c
             const int sr = s0 + b * kRound;
             raw_wait(rbar + 8u * q, (unsigned)(((b + q) / 2) & 1), status, budget);   // round b's rows
             // anchor of this round: phi reduced to [-pi, pi] (two-constant Cody-Waite
-            // split of 2 pi), __sincosf, times gain, scale and flag
+            // split of 2 pi), sine and cosine, times gain, scale and flag. FX_F32 takes
+            // sincosf: with __sincosf the eight steps from the anchor would leave the
+            // block further from FP64 than one __sincosf per channel did (20 stations
+            // x 700 spectra 3.28e-7, with anchors 3.44e-7, so 3.01e-7), and it is no slower
+            // (the 8-bit case above 5.02 -> 4.86 ms)
             float2 e;
             {
                 const float phi = fmaf((float)(TIME ? sr : sr + aj), pst.y, pst.x);
                 const float kq = rintf(phi * 0.15915494309189535f);
                 float r = fmaf(-kq, 6.28125f, phi);
                 r = fmaf(-kq, 1.9353071795864769e-3f, r);
-                __sincosf(r, &e.y, &e.x);
+                if constexpr (OUT == 1) sincosf(r, &e.y, &e.x);
+                else __sincosf(r, &e.y, &e.x);
             }
             e = cmul(gsc, e);
             if (!TIME && flags) {
