@@ -225,7 +225,9 @@ fx_status fx_channelize_correct(fx_handle *h, const void *d_raw, const double *d
  * FP64 the tensor-core form is no less accurate than the FMA chain, over all
  * baselines and over the cross baselines alone, correlated or not, while some
  * 32 or more spectra of a baseline are not zero; with fewer (lost data) its error
- * stays at about 1e-7, where the chain's falls towards 3e-8. */
+ * stays at about 1e-7, where the chain's falls towards 3e-8. With FP32 operands
+ * and up to 24 stations the order of the sums (parts of the block one after the
+ * other, or the whole) depends on the handle's subbands x channels. */
 fx_status fx_correlate(fx_handle *h, const void *d_corr, float *d_vis, fx_stream stream);
 
 /* End to end from host memory: raw samples in, visibilities out, for all
@@ -241,7 +243,9 @@ fx_status fx_correlate(fx_handle *h, const void *d_corr, float *d_vis, fx_stream
  * should be page-locked (cudaHostAlloc / cudaHostRegister) for the copies to
  * overlap. Asynchronous: `stream` waits for the whole pipeline, so
  * synchronising `stream` makes h_vis valid; the host inputs must stay
- * unchanged until then. Uses its own streams, so it is not capturable.
+ * unchanged until then. Uses its own streams, so it is not capturable. The
+ * visibilities have the bits of fx_channelize_correct + fx_correlate on the same
+ * handle, whatever host_chunk_subbands.
  * FX_ERR_INVALID if the handle was created with host_chunk_subbands = 0. */
 fx_status fx_process_host(fx_handle *h, const void *h_raw, const double *h_delay_begin,
                           const double *h_delay_end, const float *h_bandpass, const float *h_gains,

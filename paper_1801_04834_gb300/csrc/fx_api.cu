@@ -128,6 +128,7 @@ extern "C" fx_status fx_create(const fx_params *pp, fx_handle **out)
     h->p = p;
     h->p.h_subband_centre_hz = nullptr;
     h->p.h_taps = nullptr;
+    h->n_subbands_all = p.n_subbands;
     h->I = (int)I;
     h->I_pad = (int)((I + 15) / 16 * 16);
     h->S_pad = (int)((S + 63) / 64 * 64);

@@ -24,6 +24,7 @@ struct Handle {
     double *d_centres = nullptr;       // [SB]
     float2 *d_phase = nullptr;         // [SB][N][C] (phi0 mod 2pi, per-spectrum step)
     float2 *d_ratio = nullptr;         // C = 256, not FP16/BF16: [N][ceil16(S)] exp(2 pi i (fs / 16) tau_n(s))
+    int n_subbands_all = 0;            // of the handle, also in a view of some of its subbands
     int *d_status = nullptr;           // device-side error word
     int2 *d_xf32_tiles = nullptr;      // tile list of the FP32 correlator
     int xf32_ntiles = 0;

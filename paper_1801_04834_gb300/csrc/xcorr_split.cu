@@ -989,7 +989,7 @@ int t3_group(int I_pad, long long channels, int num_sms)
     return (int)std::max<long long>(1, std::min<long long>(128 / I_pad, channels / num_sms));
 }
 
-// Time segments per item where there are not even two channels per SM to group: up
+// Time segments per item where the handle has not even two channels per SM to group: up
 // to 24 stations (48 inputs), a channel's spectra in 128 / I_pad segments side by
 // side, at least four stages each, whose diagonal blocks are summed at the end (8
 // stations x 64 channels x 768 spectra: 29 us in one, 16 us in eight). More stations leave
@@ -1051,9 +1051,13 @@ cudaError_t t3_launch(const Handle &h, const void *corr, float2 *vis, cudaStream
 {
     T3Plan pl;
     const long long channels = (long long)h.p.n_subbands * h.p.n_channels;
-    const int group = t3_group(h.I_pad, channels, h.num_sms);
     const int nk = (h.p.n_spectra + kT3K - 1) / kT3K;
-    const int segs = t3_segments(h.I_pad, group, nk);
+    // Time segments change the order of the sums, so the whole handle's channels decide on
+    // them and a launch over some of its subbands gives the same bits; sharing a tile
+    // changes no sum, and goes by the launch's own channels.
+    const long long all = (long long)h.n_subbands_all * h.p.n_channels;
+    const int segs = t3_segments(h.I_pad, t3_group(h.I_pad, all, h.num_sms), nk);
+    const int group = t3_group(h.I_pad, channels, h.num_sms);
     if (!t3_plan(h.I_pad, BLOCKED, group * segs, pl)) return cudaErrorNotSupported;
     if (2 * channels > 0x7fffffffLL) return cudaErrorInvalidValue;
     T3Params P;
