@@ -59,7 +59,7 @@ cudaError_t launch_xstage(const Handle &h, const void *corr, float2 *vis, cudaSt
     case FX_F32:
         return xf32_on_tensor_cores(h) ? launch_xcorr_f32_tc(h, static_cast<const float2 *>(corr), vis, st, accumulate)
                                        : launch_xcorr_f32(h, static_cast<const float2 *>(corr), vis, st, accumulate);
-    case FX_TF32_SPLIT: return launch_xcorr_split(h, static_cast<const float *>(corr), vis, st);
+    case FX_TF32_SPLIT: return launch_xcorr_split(h, static_cast<const float *>(corr), vis, st, accumulate);
     default: return launch_xcorr_tc(h, corr, vis, st, accumulate);
     }
 }

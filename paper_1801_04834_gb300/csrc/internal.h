@@ -108,7 +108,8 @@ cudaError_t launch_beamform(const Handle &h, const void *corr, int n_beams, cons
 
 // xcorr_split.cu (FX_TF32_SPLIT, and FX_F32 where xf32_on_tensor_cores)
 bool xsplit_supported(int I_pad);
-cudaError_t launch_xcorr_split(const Handle &h, const float *corr, float2 *vis, cudaStream_t st);
+cudaError_t launch_xcorr_split(const Handle &h, const float *corr, float2 *vis, cudaStream_t st,
+                               bool accumulate = false);    // accumulate: add to vis
 bool xf32_on_tensor_cores(const Handle &h);   // FX_F32: this form rather than the CUDA-core one
 cudaError_t launch_xcorr_f32_tc(const Handle &h, const float2 *corr, float2 *vis, cudaStream_t st,
                                 bool accumulate = false);   // accumulate: add to vis

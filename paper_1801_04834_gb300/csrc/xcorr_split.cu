@@ -1130,9 +1130,9 @@ bool xsplit_supported(int I_pad)
     return t3_plan(I_pad, false, 1, pl);
 }
 
-cudaError_t launch_xcorr_split(const Handle &h, const float *corr, float2 *vis, cudaStream_t st)
+cudaError_t launch_xcorr_split(const Handle &h, const float *corr, float2 *vis, cudaStream_t st, bool accumulate)
 {
-    return t3_launch<false>(h, corr, vis, st, false, 4);   // 64 spectra per accumulator chain
+    return t3_launch<false>(h, corr, vis, st, accumulate, 4);   // 64 spectra per accumulator chain
 }
 
 // FX_F32 goes to the tensor cores where that is at least as accurate as the
