@@ -303,14 +303,15 @@ static __device__ __align__(256) float2 g_noalloc_phase[FX_NOALLOC_MAX_PHASES];
 }  // namespace
 
 cudaError_t launch_phase_table(const Handle &h, const double *tau_b, const double *tau_e,
-                               cudaStream_t st)
+                               cudaStream_t st, bool steps)
 {
+    float2 *ratio = steps ? h.d_ratio : nullptr;
     const long long n = (long long)h.p.n_subbands * h.p.n_stations * h.p.n_channels +
-                        (h.d_ratio ? (long long)h.p.n_stations * ((h.p.n_spectra + 15) / 16 * 16) : 0);
+                        (ratio ? (long long)h.p.n_stations * ((h.p.n_spectra + 15) / 16 * 16) : 0);
     const int threads = 256;
     const long long blocks = (n + threads - 1) / threads;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    phase_table_kernel<<<(unsigned)blocks, threads, 0, st>>>(h.d_centres, tau_b, tau_e, h.d_phase, h.d_ratio,
+    phase_table_kernel<<<(unsigned)blocks, threads, 0, st>>>(h.d_centres, tau_b, tau_e, h.d_phase, ratio,
                                                              h.p.n_subbands, h.p.n_stations,
                                                              h.p.n_channels, h.p.n_spectra,
                                                              h.p.sample_rate_hz, 1.0 / (double)h.p.n_spectra, 1.0 / (double)h.p.n_channels);

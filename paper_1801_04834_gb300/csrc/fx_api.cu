@@ -293,7 +293,7 @@ extern "C" fx_status fx_correct(fx_handle *h, const float *d_chan, const double 
         ((uintptr_t)d_bandpass & 3) || ((uintptr_t)d_delay_begin & 7) || ((uintptr_t)d_delay_end & 7))
         return fail(FX_ERR_INVALID, "fx_correct: misaligned buffer");
     cudaStream_t s = (cudaStream_t)stream;
-    cudaError_t e = fxi::launch_phase_table(*h, d_delay_begin, d_delay_end, s);
+    cudaError_t e = fxi::launch_phase_table(*h, d_delay_begin, d_delay_end, s, false);
     if (e == cudaSuccess)
         e = fxi::launch_correct(*h, reinterpret_cast<const float2 *>(d_chan), d_bandpass,
                                 reinterpret_cast<const float2 *>(d_gains), d_corr, s);
@@ -566,7 +566,7 @@ extern "C" fx_status fx_correct_correlate_backward_interp(
     cudaStream_t s = (cudaStream_t)stream;
     const size_t vis_len = (size_t)h->p.n_subbands * h->p.n_channels * h->B * 4;   // float2 per visibility block
     float2 *K = reinterpret_cast<float2 *>(d_work_vis), *M1 = K + vis_len;
-    cudaError_t e = fxi::launch_phase_table(*h, d_delay_begin, d_delay_end, s);
+    cudaError_t e = fxi::launch_phase_table(*h, d_delay_begin, d_delay_end, s, false);
     if (e == cudaSuccess)   // the corrected block with unit gains: Y
         e = fxi::launch_correct(*h, reinterpret_cast<const float2 *>(d_chan), d_bandpass, nullptr, d_work_corr, s);
     if (e == cudaSuccess) e = adjoint_xstage(*h, d_work_corr, K, false, s);           // K = sum Y Y^H

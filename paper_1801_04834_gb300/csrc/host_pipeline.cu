@@ -165,7 +165,7 @@ cudaError_t pipe_run(Handle &h, const void *h_raw, const double *h_tb, const dou
             v.p.n_subbands = piece;
             v.d_centres = h.d_centres + sb;
             v.d_phase = h.d_phase + sb * N * C;
-            RUN_TRY(launch_phase_table(v, P.d_tau, P.d_tau + N, P.s_comp));
+            RUN_TRY(launch_phase_table(v, P.d_tau, P.d_tau + N, P.s_comp, sb == 0));   // steps: the same for all
             RUN_TRY(launch_channelize_correct(v, d_raw, h_bp ? P.d_bp : nullptr, h_gains ? P.d_gain : nullptr, d_corr,
                                               P.s_comp));
             RUN_TRY(launch_xstage(v, d_corr, d_vis, P.s_comp));

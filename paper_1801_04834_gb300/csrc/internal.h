@@ -67,8 +67,9 @@ cudaError_t launch_stream_history(Handle &h, const void *d_new, cudaStream_t st)
 cudaError_t launch_baseline_counts(const Handle &h, const float *flags, float *counts, cudaStream_t st);
 
 // correct.cu
+// steps: also the handle's d_ratio, if it has one (what the fused F-stage reads, fx_correct does not)
 cudaError_t launch_phase_table(const Handle &h, const double *tau_b, const double *tau_e,
-                               cudaStream_t st);
+                               cudaStream_t st, bool steps = true);
 cudaError_t launch_correct(const Handle &h, const float2 *chan, const float *bandpass,
                            const float2 *gains, void *corr, cudaStream_t st);
 constexpr int kMaxDevices = 64;
