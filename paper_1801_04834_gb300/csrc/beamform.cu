@@ -624,7 +624,7 @@ cudaError_t launch_beamform(const Handle &h, const void *corr, int NB, const dou
     // blocks would not fill the SMs (7 stations, 16 beams, 64 channels, one subband:
     // the whole beam call 73 us unsplit, 62 in four)
     const unsigned wblocks = (unsigned)((wthreads + 255) / 256);
-    bf_weight_kernel<<<dim3(wblocks, wblocks < 152 ? 4 : C >= 256 ? 2 : 1), 256, 0, st>>>(
+    bf_weight_kernel<<<dim3(wblocks, wblocks < (unsigned)h.num_sms ? 4 : C >= 256 ? 2 : 1), 256, 0, st>>>(
         delays, weights, h.d_centres, h.d_bfw, SB, C, N, NB, NB_pad, h.p.sample_rate_hz, bf16);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
