@@ -224,7 +224,7 @@ fx_status fx_channelize_correct(fx_handle *h, const void *d_raw, const double *d
  * and where an FX_FLAG_XF32_* flag asks for a form of those. Normwise against
  * FP64 the tensor-core form is no less accurate than the FMA chain, over all
  * baselines and over the cross baselines alone, correlated or not, while some
- * 32 or more spectra of a baseline are not zero; with fewer (lost data) its error
+ * 50 or more spectra of a baseline are not zero; with fewer (lost data) its error
  * stays at about 1e-7, where the chain's falls towards 3e-8. With FP32 operands
  * and up to 24 stations the order of the sums (parts of the block one after the
  * other, or the whole) depends on the handle's subbands x channels. */

@@ -18,10 +18,10 @@
 //   FX_F32 takes the place of an FP32 FMA chain and may lose no more than that
 // does. hi is x rounded to TF32, so |lo| <= 2^-11 |x| with both signs; a TF32 MMA
 // reads 11 of lo's at most 12 bits (2^-24 of x RMS), and lo lo' is 2^-24 of the
-// product RMS. With BF16 cross terms, as above, the error of one product, 2^-21, showed
-// wherever a chain is short or its sum small: uncorrelated stations up to 768
-// spectra (2.3 times the chain's at 128) and lossy blocks (half of the spectra
-// lost: 4.6 times at 128, 1.9 at 768).
+// product RMS. With BF16 cross terms, as above, one product's error of 2^-21 shows
+// wherever the FMA chain is short or its sum small: uncorrelated stations below
+// 768 spectra (2.3 times the chain's error at 128) and lossy blocks (half of the
+// spectra lost: 4.6 times at 128, 1.9 at 768).
 //
 // What bounds it: shared-memory bandwidth (tensor-core operand reads plus the
 // converter's traffic), then the tensor pipe. So a diagonal tile, where row
@@ -380,11 +380,12 @@ __device__ __forceinline__ void convert_planar(unsigned char *tf, unsigned tp, u
 // Spectrum-blocked operands: `land` holds stations' runs of [16 spectra][2
 // pols] complex values; a task is 4 spectra of one station, both pols, written
 // to the FP32 planes (64-byte rows, 64-byte swizzle, pitch tp). Spectra from
-// s_lim on count as zero (every gst stations seg fewer: time segments). The four 16-byte reads of a task are rotated by
-// lane / 2 so that eight lanes' reads fall on distinct banks, and sorted again
-// in registers. Rows are ordered pol by pol within eight stations (row 16 (st /
-// 8) + 8 p + st mod 8), so that the lanes of a store take consecutive rows and
-// distinct banks too. Returns whether a value of this thread's wants SAFE.
+// s_lim on count as zero (every gst stations seg fewer: time segments). The four
+// 16-byte reads of a task are rotated by lane / 2 so that eight lanes' reads fall
+// on distinct banks, and sorted again in registers. Rows are ordered pol by pol
+// within eight stations (row 16 (st / 8) + 8 p + st mod 8), so that the lanes of a
+// store take consecutive rows and distinct banks too. Returns whether a value of
+// this thread's wants SAFE.
 template <int ROLE, bool SEG, int MODE>
 __device__ __forceinline__ bool convert_blocked(const unsigned char *land, unsigned char *tf, unsigned tp, int rows,
                                                 int s_lim, int gst, int seg, int t)
@@ -416,8 +417,10 @@ __device__ __forceinline__ bool convert_blocked(const unsigned char *land, unsig
 #pragma unroll
         for (int p = 0; p < kPols; ++p) {
             float4 hr, hj, lr, lj;
-            split4<MODE>(p ? make_float4(v[0].z, v[1].z, v[2].z, v[3].z) : make_float4(v[0].x, v[1].x, v[2].x, v[3].x), hr, lr);
-            split4<MODE>(p ? make_float4(v[0].w, v[1].w, v[2].w, v[3].w) : make_float4(v[0].y, v[1].y, v[2].y, v[3].y), hj, lj);
+            split4<MODE>(p ? make_float4(v[0].z, v[1].z, v[2].z, v[3].z)
+                           : make_float4(v[0].x, v[1].x, v[2].x, v[3].x), hr, lr);
+            split4<MODE>(p ? make_float4(v[0].w, v[1].w, v[2].w, v[3].w)
+                           : make_float4(v[0].y, v[1].y, v[2].y, v[3].y), hj, lj);
             put_tf<ROLE>(hr, hj, lr, lj, tf + tf_off(16 * (st >> 3) + 8 * p + (st & 7), lc), tp);
         }
     }
@@ -638,8 +641,9 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_split_kernel(const __grid
                                 if constexpr (BLOCKED) {
 #pragma unroll
                                     for (int kk = 0; kk < kT3K / 8; ++kk) {
-                                        mma_tf32(d, tf + tp + 2u * kk, tf + 2 * tp + 2u * kk, id2, (kc | kk) ? 1u : 0u);   // hJ x [lR; 2lJ]
-                                        mma_tf32(d, tf + 2u * kk, tf + 4 * tp + 2u * kk, id2, 1u);                         // hR x [-lJ; 2lR]
+                                        const unsigned long long t = tf + 2u * kk;
+                                        mma_tf32(d, t + tp, t + 2 * tp, id2, (kc | kk) ? 1u : 0u);   // hJ x [lR; 2lJ]
+                                        mma_tf32(d, t, t + 4 * tp, id2, 1u);                         // hR x [-lJ; 2lR]
                                     }
                                 } else {
                                     mma_f16(d, bf + bp, bf + 2 * bp, idb, kc ? 1u : 0u);             // hJ x [lR; 2lJ]
@@ -734,7 +738,8 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_split_kernel(const __grid
                         auto convert = [&](auto mode) {
                             constexpr int MODE = decltype(mode)::value;
                             if (diag) return convert_blocked<DIAG, SEG, MODE>(la, st, pitch, n, lim, gst, seg, ct);
-                            const bool rows = convert_blocked<ROWS, false, MODE>(la + P.row_land, st, TA, 128, lim, gst, seg, ct);
+                            const bool rows =
+                                convert_blocked<ROWS, false, MODE>(la + P.row_land, st, TA, 128, lim, gst, seg, ct);
                             return convert_blocked<COLS, false, MODE>(la, st + 4 * TA, pitch, n, lim, gst, seg, ct) || rows;
                         };
                         // An infinity meets every other station's lo parts, which other warps of the
@@ -827,14 +832,20 @@ __global__ void __launch_bounds__(kT3Threads, 1) xcorr_split_kernel(const __grid
                 // on or below the diagonal into the scratch and reads the mirror
                 // blocks of those on or above it (rows of 33 words: no bank
                 // conflicts), all ten blocks at once or, with less scratch, the diagonal
-                // ones last, after six others at once or three and three. Channels or
-                // segments of up to 32 inputs need the diagonal blocks only.
-                const bool small = P.gin <= 32;
-                const int phases = small || P.scratch_bytes >= kT3Scratch ? 1 : P.scratch_bytes >= kT3ScratchMid ? 2 : 3;
+                // ones last, after three and three others or (blocked) six at once. Blocked
+                // channels or segments of up to 32 inputs pass the diagonal ones only.
+                const bool diag_only = BLOCKED && P.gin <= 32;
+                const int phases = diag_only || P.scratch_bytes >= kT3Scratch     ? 1
+                                   : BLOCKED && P.scratch_bytes >= kT3ScratchMid ? 2
+                                                                                 : 3;
                 auto place = [&](int r, int c, int &slot) {     // block (r, c), c <= r: phase and slot
-                    const int o = r * (r - 1) / 2 + c;          // rank among those below the diagonal
-                    slot = r == c ? r : phases == 1 ? 4 + o : phases == 2 ? o : o % 3;
-                    return r == c ? phases - 1 : small ? -1 : phases == 3 ? o / 3 : 0;
+                    if (!diag_only && phases == 1) {
+                        slot = r * (r + 1) / 2 + c;
+                        return 0;
+                    }
+                    const int o = r * (r - 1) / 2 + c;
+                    slot = r == c ? r : phases == 2 ? o : o % 3;
+                    return r == c ? phases - 1 : diag_only ? -1 : phases == 2 ? 0 : o / 3;
                 };
                 auto put = [&](const float2 (&A)[32], int phase) {
 #pragma unroll
@@ -981,7 +992,7 @@ EncodeTiledFn t3_encode_fn()
 // takes about the same time (0.45 us with 16 inputs, 0.6 us with 128), so small
 // arrays share one: G channels' inputs side by side, of whose products only the
 // G diagonal blocks are written. As many as fit while every SM still gets an item
-// (15616 channels x 256 spectra of 8 stations: blocked 1.10 ms alone, 0.23 ms in
+// (15616 channels x 256 spectra of 8 stations: blocked 1.10 ms alone, 0.24 ms in
 // eights, planar 0.77 and 0.15 ms).
 int t3_group(int I_pad, long long channels, int num_sms)
 {
@@ -1144,12 +1155,13 @@ cudaError_t launch_xcorr_split(const Handle &h, const float *corr, float2 *vis, 
 //   uncorrelated noise            0.74 0.46   0.46 0.30   0.35 0.24   0.56 0.37   0.37 0.24
 //   with a common signal          0.65 0.44   0.37 0.27   0.26 0.21   0.49 0.39   0.26 0.23
 //   half of the spectra lost      0.86 0.80   0.59 0.54   0.44 0.44   0.63 0.56   0.43 0.37
-// Chains of 32 would have up to 1.7 at 128 spectra and 1.2 at 384 (half lost); they drain
-// the accumulator half as often (64 stations x 1280 channels x 1024 spectra 476 us,
-// with 16 583, CUDA cores 2056). What the chain length cannot mend is a baseline
-// with few live spectra, where an FMA chain barely rounds: 64 live spectra 0.9 0.8
-// of its error, 16 1.2 1.2, 4 2.1 2.0, one 3.4 3.3 (1e-7 of the product). Shorter integrations and the
-// forms asked for by flag stay on the CUDA cores.
+// Chains of 32 would have up to 1.7 at 128 spectra and 1.2 at 384 (half lost); they
+// drain the accumulator half as often (64 stations x 1280 channels x 1024 spectra
+// 476 us, with 16 583, CUDA cores 2056). What the chain length cannot mend is a
+// baseline with few live spectra, where an FMA chain barely rounds: with 64 of them
+// 0.9 and 0.8 of its error, with 16 1.2 and 1.2, 4 2.1 and 2.0, one 3.4 and 3.3
+// (1e-7 of the product). Shorter integrations and the forms asked for by flag stay
+// on the CUDA cores.
 constexpr int kXf32TcSpectra = 128;
 
 bool xf32_on_tensor_cores(const Handle &h)
