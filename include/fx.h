@@ -219,8 +219,8 @@ fx_status fx_channelize_correct(fx_handle *h, const void *d_raw, const double *d
  * with FP32 accumulation, accumulator chains of 64 spectra summed in IEEE FP32
  * (FP32 accuracy, any station count up to 512; results reproducible run to
  * run). FX_F32 operands run there from 128 spectra on, with hi rounded and the
- * cross terms in TF32 too (chains of 16 spectra, 32 from 1024 on; reproducible
- * likewise), and as FP32 FMAs on the CUDA cores below that, above 512 stations,
+ * cross terms in TF32 too (chains of 16 spectra, 32 from 768 or 1024 on;
+ * reproducible likewise), and as FP32 FMAs on the CUDA cores below that, above 512 stations,
  * and where an FX_FLAG_XF32_* flag asks for a form of those. Normwise against
  * FP64 the tensor-core form is no less accurate than the FMA chain, over all
  * baselines and over the cross baselines alone, correlated or not, while some

@@ -1151,13 +1151,15 @@ cudaError_t launch_xcorr_split(const Handle &h, const float *corr, float2 *vis, 
 // baselines normwise / over the cross baselines, error as a multiple of the
 // chain's (8, 50 and 76 stations; the chain has 2.4e-7 at 128 spectra, 4e-7 at 384,
 // 6e-7 at 768, 1.2e-6 at 3072):
-//   spectra (accumulator chain)    128 (16)    384 (16)    768 (16)    1024 (32)   3072 (32)
-//   uncorrelated noise            0.74 0.46   0.46 0.30   0.35 0.24   0.56 0.37   0.37 0.24
-//   with a common signal          0.65 0.44   0.37 0.27   0.26 0.21   0.49 0.39   0.26 0.23
-//   half of the spectra lost      0.86 0.80   0.59 0.54   0.44 0.44   0.63 0.56   0.43 0.37
-// Chains of 32 would have up to 1.7 at 128 spectra and 1.2 at 384 (half lost); they
-// drain the accumulator half as often (64 stations x 1280 channels x 1024 spectra
-// 476 us, with 16 583, CUDA cores 2056). What the chain length cannot mend is a
+//   spectra (accumulator chain)    128 (16)    384 (16)    768 (16)    768 (32)   1024 (32)   3072 (32)
+//   uncorrelated noise            0.74 0.46   0.46 0.30   0.35 0.24   0.73 0.43   0.56 0.37   0.37 0.24
+//   with a common signal          0.65 0.44   0.37 0.27   0.26 0.21   0.53 0.41   0.49 0.39   0.26 0.23
+//   half of the spectra lost      0.86 0.80   0.59 0.54   0.44 0.44   0.79 0.63   0.63 0.56   0.43 0.37
+// So chains of 32 from 768 spectra on, or from 1024 on where autocorrelations, which
+// lose most to a longer chain, are most of the norm (up to 32 stations); at 128
+// spectra they would have up to 1.7, at 384 1.2 (half lost). They drain the
+// accumulator half as often (64 stations x 1280 channels x 1024 spectra 476 us,
+// with 16 583, CUDA cores 2056). What the chain length cannot mend is a
 // baseline with few live spectra, where an FMA chain barely rounds: with 64 of them
 // 0.9 and 0.8 of its error, with 16 1.2 and 1.2, 4 2.1 and 2.0, one 3.4 and 3.3
 // (1e-7 of the product). Shorter integrations and the forms asked for by flag stay
@@ -1173,7 +1175,7 @@ bool xf32_on_tensor_cores(const Handle &h)
 
 cudaError_t launch_xcorr_f32_tc(const Handle &h, const float2 *corr, float2 *vis, cudaStream_t st, bool accumulate)
 {
-    return t3_launch<true>(h, corr, vis, st, accumulate, h.p.n_spectra >= 1024 ? 2 : 1);
+    return t3_launch<true>(h, corr, vis, st, accumulate, h.p.n_spectra >= (h.I_pad > 64 ? 768 : 1024) ? 2 : 1);
 }
 
 }  // namespace fxi

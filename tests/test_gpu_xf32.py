@@ -61,7 +61,7 @@ def operands(kind, N, C, S):
 
 
 @pytest.mark.parametrize("N", [8, 50, 76])            # time segments, one tile, off-diagonal tiles
-@pytest.mark.parametrize("S", [128, 383, 384, 1023, 1024, 1536])
+@pytest.mark.parametrize("S", [128, 383, 384, 768, 1023, 1024, 1536])
 @pytest.mark.parametrize("kind", ["noise", "common", "half"])
 def test_no_less_accurate_than_the_fma_chain(N, S, kind):
     """Normwise over all baselines, over the cross baselines alone (whose sums are small
