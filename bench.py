@@ -12,7 +12,8 @@ per-station bandpass ripple, 16-tap PPF to 64 channels, 3072 spectra per block
 (1.00663 s of sky), FP32-accurate path: the X-stage runs on the tcgen05 tensor
 cores with each FP32 operand split into hi + lo, hi hi' as TF32 MMAs and the
 cross terms hi lo' + lo hi' as BF16 MMAs (FX_TF32_SPLIT).
-The default precision (FX_F32, the same split on the spectrum-blocked layout),
+The default precision (FX_F32, the same split on the spectrum-blocked layout,
+every term as TF32 MMAs),
 the CUDA-core FFMA FP32 X-stage and the FP16 / BF16 / split-FP16 tensor-core
 X-stages are timed on the same block, and the 8-bit precision workload (64
 stations, 488 subbands, 256 channels, 768 spectra) is timed at its own shape;
@@ -119,8 +120,8 @@ def executed_xflops_split(c, w):
 
 
 def executed_xflops_half(c, w):
-    """(TF32, BF16) tensor-core flops the FP32-accurate X-stage issues: as
-    executed_xflops_split off the diagonal; a diagonal item of n inputs forms
+    """(TF32, BF16) tensor-core flops the FP32-accurate X-stage issues (FX_F32:
+    the second figure in TF32 too): as executed_xflops_split off the diagonal; a diagonal item of n inputs forms
     3 of the 4 real products of hi hi' and one of the two cross terms."""
     t = b = 0
     for row0 in range(0, c.I_pad, 128):
@@ -539,16 +540,19 @@ def run_fx(args, w):
     if prec in (0, 4):
         ex = executed_xflops_half(c, w)
         tpk, bpk = peaks_run["tf32_tflops"], peaks_run["bf16_tflops"]
+        cross = "BF16"
+        if prec == 0:                                 # FX_F32: the cross terms are TF32 MMAs too
+            bpk, cross = tpk, "TF32"
         sr = split_roofline(xflops, ex, ms_x, tpk, bpk)
         roof = {"kernel": "xcorr_split_kernel", "bound": "tensor", "achieved": sr["achieved"], "peak": tpk,
                 "unit": "TFLOP/s", "frac": sr["frac"],
                 "traffic": recorded_traffic("xcorr_split_kernel", args.workload),
                 "peak_source": "dense TF32 tensor throughput measured in this run (torch TF32 matmul 8192^3, "
-                               "burst); MEASURED_PEAKS.json holds no TF32 figure; BF16 peak of the same run "
-                               f"({bpk:.0f} TFLOP/s) for the BF16 part",
-                "algorithmic": f"{xflops:.4e} TF32 flop (hi hi') + {2 * xflops:.4e} BF16 flop (hi lo' + lo hi') "
+                               "burst); MEASURED_PEAKS.json holds no TF32 figure; "
+                               f"{cross} peak of the same run ({bpk:.0f} TFLOP/s) for the cross terms",
+                "algorithmic": f"{xflops:.4e} TF32 flop (hi hi') + {2 * xflops:.4e} {cross} flop (hi lo' + lo hi') "
                                f"per launch, 8 flop per complex MAC and product, upper triangle incl. autos; "
-                               f"achieved in TF32-equivalent flops (BF16 x P_tf32/P_bf16), frac = "
+                               f"achieved in TF32-equivalent flops (cross terms x P_tf32/P_{cross.lower()}), frac = "
                                f"floor {sr['floor_ms']:.2f} ms / measured {ms_x:.2f} ms",
                 "useful_fp32_equiv_TFLOPs": x_ach, "useful_frac": x_ach / tpk,
                 "executed_TFLOPs": sr["executed_TFLOPs"], "executed_frac": sr["executed_frac"],

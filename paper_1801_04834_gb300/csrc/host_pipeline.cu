@@ -147,7 +147,8 @@ cudaError_t pipe_run(Handle &h, const void *h_raw, const double *h_tb, const dou
         // subband where a subband is long enough to upload (8 MB, some 40 us, against the
         // launches of a piece): nothing is left to hide its computation behind, so only
         // one subband's stands after the last upload (64 stations x 8 subbands x 3072
-        // spectra of int16 in chunks of 4: 4.53 -> 4.15 ms, 4.0 of it the link).
+        // spectra of int16 in chunks of 4, over a link of 200 GB/s: 4.61 -> 4.16 ms, 4.0 of
+        // it the link; a link of half that, or an unsteady one, hides the gain).
         if (k >= 2) RUN_TRY(cudaStreamWaitEvent(P.s_in, P.comp_done[b], 0));
         if (k >= 2) RUN_TRY(cudaStreamWaitEvent(P.s_comp, P.out_done[b], 0));
         const int piece = k == nch - 1 && P.raw_sb >= kPieceBytes ? 1 : cs;

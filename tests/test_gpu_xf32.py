@@ -140,3 +140,20 @@ def test_cuda_core_form_at_any_length(N, S):
     assert not torch.equal(vis["4x4"], vis["auto"])   # the default is another form at this length
     ref = product(y)
     assert ((vis["4x4"].double() - ref).norm() / ref.norm()).item() < S * 2.0 ** -24
+
+
+def test_cuda_core_form_full_shape_sampled():
+    """The CUDA-core form at the LOFAR shape (64 stations, 10 subbands, 64 channels, 3072 spectra:
+    256-thread blocks, 32-spectrum chunks) on sampled channels, held to the FP32 path's bound."""
+    import paper_1801_04834_gb300 as m
+    N, SB, C, S = 64, 10, 64, 3072
+    c = correlator(N, SB, C, S, xf32_form="4x4")
+    g = torch.Generator(device="cuda")
+    g.manual_seed(180104834)
+    corr = torch.randn(c.corr_shape(), generator=g, device="cuda") * 30
+    vis = c.correlate(corr)
+    y = m.f32_unblock(corr, S)
+    for sb, k in ((0, 0), (4, 31), (9, 63)):
+        ref = product(y[sb:sb + 1, k:k + 1].contiguous())[0, 0]
+        assert ((vis[sb, k].double() - ref).norm() / ref.norm()).item() < 1e-5
+    c.close()
